@@ -332,12 +332,12 @@ __device__ __forceinline__ Setup setup_sample(const SampleArgs& a, SampleStream&
 }
 
 // One level of the bound-driven descent below internal node `node` (ud: the
-// level's draw; x*: the shading point, n*: its normal broadcast to both
-// components). Both children's bounds in one packed evaluation; they are
+// level's draw; nx*: the shading point negated, n*: its normal, broadcast to
+// both components). Both children's bounds in one packed evaluation; they are
 // compared without a division: w_L = num_L den_R, w_R = num_R den_L; their
 // powers if both vanish.
 __device__ __forceinline__ void descent_step(const SampleArgs& a, uint32_t& node, float& p_in, float ud,
-                                             float x0, float x1, float x2, float2 n0, float2 n1, float2 n2)
+                                             float2 nx0, float2 nx1, float2 nx2, float2 n0, float2 n1, float2 n2)
 {
     PairRec q;
     {
@@ -346,9 +346,9 @@ __device__ __forceinline__ void descent_step(const SampleArgs& a, uint32_t& node
 #pragma unroll
         for (int k = 0; k < 5; ++k) dst[k] = __ldg(src + k);
     }
-    const Bound2 b = importance2(q, x0, x1, x2, n0, n1, n2);
-    const float2 w = __fmul2_rn(b.num, make_float2(b.den.y, b.den.x));
-    float wl = w.x, wr = w.y;
+    const NodePair np{q.c0, q.c1, q.c2, q.r, q.a0, q.a1, q.a2, q.cs.x, q.cs.y};
+    const Bound2 b = importance2(np, q.phi, nx0, nx1, nx2, n0, n1, n2);
+    float wl = fmul(b.num.x, b.den.y), wr = fmul(b.num.y, b.den.x);
     float ssum = fadd(wl, wr);
     if (!(ssum > 0.0f)) {
         wl = q.phi.x;
@@ -480,19 +480,20 @@ __device__ __forceinline__ void sample_point(const SampleArgs& a, int64_t p, con
             light = leaf_or_flag(a, node, nl1);
         } else {
             const float2 vn0 = make_float2(n0, n0), vn1 = make_float2(n1, n1), vn2 = make_float2(n2, n2);
+            const float2 vx0 = make_float2(-x0, -x0), vx1 = make_float2(-x1, -x1), vx2 = make_float2(-x2, -x2);
             // level l takes draw kDrawDescent + l: words 1..3 of Philox block 2, then four levels per
             // block, unrolled so that every word index is a constant
             static_assert(kDrawDescent == 9, "descent draws start at word 1 of block 2");
             uint4 w = rs.block_words(2);
-            if (node < nl1u) descent_step(a, node, p_in, u24(w.y), x0, x1, x2, vn0, vn1, vn2);
-            if (node < nl1u) descent_step(a, node, p_in, u24(w.z), x0, x1, x2, vn0, vn1, vn2);
-            if (node < nl1u) descent_step(a, node, p_in, u24(w.w), x0, x1, x2, vn0, vn1, vn2);
+            if (node < nl1u) descent_step(a, node, p_in, u24(w.y), vx0, vx1, vx2, vn0, vn1, vn2);
+            if (node < nl1u) descent_step(a, node, p_in, u24(w.z), vx0, vx1, vx2, vn0, vn1, vn2);
+            if (node < nl1u) descent_step(a, node, p_in, u24(w.w), vx0, vx1, vx2, vn0, vn1, vn2);
             for (uint32_t b = 3; node < nl1u && b < (uint32_t)(kMaxTreeDepth / 4); ++b) {
                 w = rs.block_words(b);
-                descent_step(a, node, p_in, u24(w.x), x0, x1, x2, vn0, vn1, vn2);
-                if (node < nl1u) descent_step(a, node, p_in, u24(w.y), x0, x1, x2, vn0, vn1, vn2);
-                if (node < nl1u) descent_step(a, node, p_in, u24(w.z), x0, x1, x2, vn0, vn1, vn2);
-                if (node < nl1u) descent_step(a, node, p_in, u24(w.w), x0, x1, x2, vn0, vn1, vn2);
+                descent_step(a, node, p_in, u24(w.x), vx0, vx1, vx2, vn0, vn1, vn2);
+                if (node < nl1u) descent_step(a, node, p_in, u24(w.y), vx0, vx1, vx2, vn0, vn1, vn2);
+                if (node < nl1u) descent_step(a, node, p_in, u24(w.z), vx0, vx1, vx2, vn0, vn1, vn2);
+                if (node < nl1u) descent_step(a, node, p_in, u24(w.w), vx0, vx1, vx2, vn0, vn1, vn2);
             }
             light = leaf_or_flag(a, node, nl1);
         }
