@@ -55,6 +55,8 @@ void free_tree(rll_tree* t)
     if (!t) return;
     cudaFree(t->nodes);
     cudaFree(t->pairs);
+    if (t->tail_tex) cudaDestroyTextureObject(t->tail_tex);
+    cudaFree(t->tails);
     cudaFree(t->quads);
     cudaFree(t->lights);
     cudaFree(t->perm);

@@ -495,6 +495,7 @@ int rll_batch_set_items(rll_ctx* ctx, rll_batch* b, const rll_batch_item* items,
         a.jitter = g->p.jitter;
         a.reward_mode = g->p.reward_mode;
         a.pairs = t->pairs;
+        a.tail_tex = t->tail_tex;
         a.quads = t->quads;
         a.nodes = t->nodes;
         a.lights = t->lights;

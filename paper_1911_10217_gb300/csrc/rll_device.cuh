@@ -60,21 +60,33 @@ struct __align__(16) DescRec {
 static_assert(sizeof(DescRec) == 48, "DescRec must be 48 bytes");
 
 // The DescRec fields of both children of one internal node, interleaved
-// (x: left child, y: right child) so that each 16-byte load yields two packed
-// operands of the paired bound below; 80 bytes per descent level (the
-// descent is bound by how many record bytes a level pulls through L1). r2 is
-// r r, formed at use; cs holds (1 - cos theta, sin theta) of each child as two
-// binary16 values (exactly the DescRec values; cos theta = 1 - v is exact).
-struct __align__(16) PairRec {
-    float2 c0, c1, c2, r, phi;
+// (x: left child, y: right child) so that a load yields packed operands of
+// the paired bound below: 64 bytes of geometry, two 256-bit loads, and 16
+// bytes of powers and ids in an array of their own. r2 is r r, formed at use;
+// cs holds (1 - cos theta, sin theta) of each child as two binary16 values
+// (exactly the DescRec values; cos theta = 1 - v is exact).
+// The sampling kernel was bound by the L1's gather rate: a divergent load
+// costs about a cycle per distinct 32-byte sector and instruction (measured
+// with 32 random records a warp: 123 cycles as five 16-byte loads of one
+// 80-byte record, 107 as 64 + 16 bytes with 256-bit loads), and its load pipe
+// was 89 % busy. The powers and ids go through the texture path, whose data
+// stage works beside the load pipe (85 -> 75 % busy). 1080p sampling 395 us
+// (80-byte records) -> 382 (wide loads) -> 359 (and the texture path); 4K
+// bfloat16 1 850 -> 1 764 -> 1 667 us.
+struct __align__(32) PairRec {
+    float2 c0, c1, c2, r;
     float2 a0, a1, a2;
     uint2 cs;
-    uint2 id;
 };
-static_assert(sizeof(PairRec) == 80, "PairRec must be 80 bytes");
+static_assert(sizeof(PairRec) == 64, "PairRec must be 64 bytes");
+struct __align__(16) PairTail {
+    float phi[2];
+    uint32_t id[2];
+};
+static_assert(sizeof(PairTail) == 16, "PairTail must be 16 bytes");
 
-// Sorted light, 64 bytes.
-struct __align__(16) LightRec {
+// Sorted light, 64 bytes (two 256-bit loads).
+struct __align__(32) LightRec {
     float v0[3];
     float v1[3];
     float v2[3];
@@ -90,6 +102,20 @@ __device__ __forceinline__ float fsub(float a, float b) { return __fsub_rn(a, b)
 __device__ __forceinline__ float fmul(float a, float b) { return __fmul_rn(a, b); }
 __device__ __forceinline__ float fdiv(float a, float b) { return __fdiv_rn(a, b); }
 __device__ __forceinline__ float fsqrt(float a) { return __fsqrt_rn(a); }
+
+// 32 bytes by one load instruction (p 32-byte aligned, not written while the kernel runs)
+struct __align__(32) Words8 {
+    uint32_t w[8];
+};
+__device__ __forceinline__ Words8 ldg_words8(const void* p)
+{
+    Words8 v;
+    asm("ld.global.nc.v8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+        : "=r"(v.w[0]), "=r"(v.w[1]), "=r"(v.w[2]), "=r"(v.w[3]), "=r"(v.w[4]), "=r"(v.w[5]), "=r"(v.w[6]),
+          "=r"(v.w[7])
+        : "l"(p));
+    return v;
+}
 
 // ---------------------------------------------------------------- Philox
 // Philox4x32-10 (Salmon et al., SC'11): 10 rounds, multipliers 0xD2511F53 and

@@ -13,6 +13,7 @@ namespace rll {
 struct NodeRec;
 struct DescRec;
 struct PairRec;
+struct PairTail;
 struct LightRec;
 }  // namespace rll
 
@@ -47,7 +48,9 @@ struct rll_tree {
     int device = 0;
     int64_t n = 0;
     rll::NodeRec* nodes = nullptr;   // [2n-1] every node
-    rll::PairRec* pairs = nullptr;   // [n-1] descent records of both children of internal i, interleaved
+    rll::PairRec* pairs = nullptr;   // [n-1] geometry of both children of internal i, interleaved
+    rll::PairTail* tails = nullptr;  // [n-1] their powers and ids
+    cudaTextureObject_t tail_tex = 0; // tails as float4 texels (n > 1)
     rll::DescRec* quads = nullptr;   // [4(n-1)] records of the 2..4 grandchildren of internal i at 4i.. (two-level
                                      // descent; a single-light child stands for itself; unused entries id ~0)
     rll::LightRec* lights = nullptr; // [n] sorted lights

@@ -5,7 +5,7 @@
 // in shared memory once per block. Per sample:
 //   hash lookup / lazy insert of the (jittered) 5-d cell   (64-bit CAS)
 //   binary search of the cell's C for the cluster s        (log2 m loads of one row)
-//   in-cluster choice: bound-driven descent (one 80-byte record of both
+//   in-cluster choice: bound-driven descent (a 64 + 16-byte record of both
 //   children per level, both bounds in packed f32x2 arithmetic) or a uniform
 //   pick over the cluster's lights
 //   uniform point on the light triangle, contribution, shadow segment vs the
@@ -185,6 +185,7 @@ int sample_and_shade_range(rll_ctx* ctx, rll_grid* g, const rll_tree* t, const f
     a.jitter = g->p.jitter;
     a.reward_mode = g->p.reward_mode;
     a.pairs = t->pairs;
+    a.tail_tex = t->tail_tex;
     a.quads = t->quads;
     a.nodes = t->nodes;
     a.lights = t->lights;

@@ -39,6 +39,7 @@ struct SampleArgs {
     uint32_t jitter;
     uint32_t reward_mode;
     const PairRec* pairs;
+    cudaTextureObject_t tail_tex;  // the pairs' powers and ids
     const DescRec* quads;     // two-level descent records (4 per internal node)
     const NodeRec* nodes;
     const LightRec* lights;
@@ -103,10 +104,9 @@ __device__ __forceinline__ DescRec load_desc(const DescRec* p)
 __device__ __forceinline__ LightRec load_light(const LightRec* p)
 {
     LightRec r;
-    const float4* s = reinterpret_cast<const float4*>(p);
-    float4* d = reinterpret_cast<float4*>(&r);
-#pragma unroll
-    for (int k = 0; k < 4; ++k) d[k] = __ldg(s + k);
+    Words8* d = reinterpret_cast<Words8*>(&r);
+    d[0] = ldg_words8(p);
+    d[1] = ldg_words8(reinterpret_cast<const char*>(p) + 32);
     return r;
 }
 
@@ -339,20 +339,18 @@ __device__ __forceinline__ Setup setup_sample(const SampleArgs& a, SampleStream&
 __device__ __forceinline__ void descent_step(const SampleArgs& a, uint32_t& node, float& p_in, float ud,
                                              float2 nx0, float2 nx1, float2 nx2, float2 n0, float2 n1, float2 n2)
 {
-    PairRec q;
-    {
-        const float4* src = reinterpret_cast<const float4*>(a.pairs + node);
-        float4* dst = reinterpret_cast<float4*>(&q);
-#pragma unroll
-        for (int k = 0; k < 5; ++k) dst[k] = __ldg(src + k);
-    }
-    const NodePair np{q.c0, q.c1, q.c2, q.r, q.a0, q.a1, q.a2, q.cs.x, q.cs.y};
-    const Bound2 b = importance2(np, q.phi, nx0, nx1, nx2, n0, n1, n2);
+    const float4 t = tex1Dfetch<float4>(a.tail_tex, (int)node);  // powers, then ids
+    const Words8 u = ldg_words8(a.pairs + node), v = ldg_words8(reinterpret_cast<const char*>(a.pairs + node) + 32);
+    auto pair = [](const Words8& w, int k) {
+        return make_float2(__uint_as_float(w.w[2 * k]), __uint_as_float(w.w[2 * k + 1]));
+    };
+    const NodePair q{pair(u, 0), pair(u, 1), pair(u, 2), pair(u, 3), pair(v, 0), pair(v, 1), pair(v, 2), v.w[6], v.w[7]};
+    const Bound2 b = importance2(q, make_float2(t.x, t.y), nx0, nx1, nx2, n0, n1, n2);
     float wl = fmul(b.num.x, b.den.y), wr = fmul(b.num.y, b.den.x);
     float ssum = fadd(wl, wr);
     if (!(ssum > 0.0f)) {
-        wl = q.phi.x;
-        wr = q.phi.y;
+        wl = t.x;
+        wr = t.y;
         ssum = fadd(wl, wr);
     }
     bool left;
@@ -365,7 +363,7 @@ __device__ __forceinline__ void descent_step(const SampleArgs& a, uint32_t& node
         ratio = 0.5f;
     }
     p_in *= ratio;
-    node = left ? q.id.x : q.id.y;
+    node = __float_as_uint(left ? t.z : t.w);
 }
 
 __device__ __forceinline__ void prefetch_l1(const void* p)

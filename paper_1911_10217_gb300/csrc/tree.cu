@@ -265,7 +265,8 @@ __global__ void k_finalize(int64_t nn, NodeRec* __restrict__ nodes, const int* _
 }
 
 __global__ void k_pairs(int64_t n, const NodeRec* __restrict__ nodes, const int32_t* __restrict__ left,
-                        const int32_t* __restrict__ right, PairRec* __restrict__ pairs, float* __restrict__ leaf_phi)
+                        const int32_t* __restrict__ right, PairRec* __restrict__ pairs, PairTail* __restrict__ tails,
+                        float* __restrict__ leaf_phi)
 {
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i < n - 1) {
@@ -275,7 +276,6 @@ __global__ void k_pairs(int64_t n, const NodeRec* __restrict__ nodes, const int3
         q.c1 = make_float2(L.c[1], R.c[1]);
         q.c2 = make_float2(L.c[2], R.c[2]);
         q.r = make_float2(L.r, R.r);
-        q.phi = make_float2(L.phi, R.phi);
         q.a0 = make_float2(L.axis[0], R.axis[0]);
         q.a1 = make_float2(L.axis[1], R.axis[1]);
         q.a2 = make_float2(L.axis[2], R.axis[2]);
@@ -284,8 +284,8 @@ __global__ void k_pairs(int64_t n, const NodeRec* __restrict__ nodes, const int3
             const __half2 hr = __halves2half2(__float2half_rn(fsub(1.0f, R.cos_t)), __float2half_rn(R.sin_t));
             q.cs = make_uint2(*reinterpret_cast<const uint32_t*>(&hl), *reinterpret_cast<const uint32_t*>(&hr));
         }
-        q.id = make_uint2(L.id, R.id);
         pairs[i] = q;
+        tails[i] = PairTail{{L.phi, R.phi}, {L.id, R.id}};
     }
     if (i < n) leaf_phi[i] = nodes[n - 1 + i].phi;
 }
@@ -621,6 +621,7 @@ int build_tree(rll_ctx* ctx, const float* tri, const float* emission, int64_t n,
     if (e != cudaSuccess) return check_cuda(ctx, e, "cudaMalloc(tree)");
     RLL_ALLOC(t->nodes, sizeof(NodeRec) * nn);
     RLL_ALLOC(t->pairs, sizeof(PairRec) * (n - 1));
+    RLL_ALLOC(t->tails, sizeof(PairTail) * (n - 1));
     RLL_ALLOC(t->quads, sizeof(DescRec) * 4 * (n - 1));
     RLL_ALLOC(t->lights, sizeof(LightRec) * n);
     RLL_ALLOC(t->perm, sizeof(uint32_t) * n);
@@ -629,6 +630,17 @@ int build_tree(rll_ctx* ctx, const float* tri, const float* emission, int64_t n,
     RLL_ALLOC(t->parent, sizeof(int32_t) * nn);
     RLL_ALLOC(t->light_cdf, sizeof(float) * n);
 #undef RLL_ALLOC
+    if (n > 1) {
+        cudaResourceDesc res{};
+        res.resType = cudaResourceTypeLinear;
+        res.res.linear.devPtr = t->tails;
+        res.res.linear.desc = cudaCreateChannelDesc<float4>();
+        res.res.linear.sizeInBytes = sizeof(PairTail) * (size_t)(n - 1);
+        cudaTextureDesc tex{};
+        tex.readMode = cudaReadModeElementType;
+        e = cudaCreateTextureObject(&t->tail_tex, &res, &tex, nullptr);
+        if (e != cudaSuccess) return check_cuda(ctx, e, "texture (tree)");
+    }
     // scratch: codes, idx, sort, begin/end (unused after build), axis sums,
     // counters, cone minima, bbox, scan sums
     const size_t sort_b = radix_sort_scratch_bytes(n);
@@ -698,7 +710,8 @@ int build_tree(rll_ctx* ctx, const float* tri, const float* emission, int64_t n,
     k_axis<<<grid_for(nn), kBlock, 0, s>>>(nn, t->nodes, axis_sum, cosmin);
     k_cone<<<grid_for(n), kBlock, 0, s>>>(n, t->lights, t->nodes, t->parent, cosmin);
     k_finalize<<<grid_for(nn), kBlock, 0, s>>>(nn, t->nodes, cosmin);
-    k_pairs<<<grid_for(n), kBlock, 0, s>>>(n, t->nodes, t->left, t->right, t->pairs, leaf_phi);
+    k_pairs<<<grid_for(n), kBlock, 0, s>>>(n, t->nodes, t->left, t->right, t->pairs, t->tails,
+                                        leaf_phi);
     if (n > 1) k_quads<<<grid_for(n - 1), kBlock, 0, s>>>(n, t->nodes, t->left, t->right, t->quads);
     e = inclusive_scan_f32(s, leaf_phi, t->light_cdf, n, scan_ws);
     if (e != cudaSuccess) return check_cuda(ctx, e, "scan (light cdf)");
