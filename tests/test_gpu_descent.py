@@ -54,3 +54,14 @@ def test_bounds_at_small_scales(env, mode, log2_scale):
     s = dataclasses.replace(s, tris=s.tris * k, boxes=s.boxes * k, pos=s.pos * k,
                             grid=dataclasses.replace(s.grid, cell_size=float(s.grid.cell_size * k)))
     check(env, s, mode=mode)
+
+
+@pytest.mark.parametrize("points,spp", [(1, 2), (37, 3), (33, 31), (5, 32), (7, 33), (3, 48), (2, 65), (1, 1000),
+                                        (4096, 2), (1000, 5)])
+def test_samples_split_over_lanes(env, points, spp):
+    """More than one sample a point: a lane a sample, points summed across lanes and rounds. Samples a
+    point that do and do not divide a warp, points that do not fill one, sums over several rounds."""
+    s = scenes.tiny_scene()
+    s = dataclasses.replace(s, pos=np.ascontiguousarray(s.pos[:, :points]), nrm=np.ascontiguousarray(s.nrm[:, :points]),
+                            albedo=s.albedo[:points])
+    check(env, s, spp=spp)
