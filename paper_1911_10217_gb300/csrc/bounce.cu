@@ -2,8 +2,8 @@
 // ingredient: the cells of a path vertex are sized from its ray footprint,
 // derived from the vertex's area pdf).
 //
-// One thread per shading point x (unit normal n), occluder boxes staged in
-// shared memory once per block:
+// One thread per shading point x (unit normal n), occluder boxes and their
+// table (box_bins.cuh) staged in shared memory once per block:
 //   a uniform point (a, b) of the unit disk by rejection from the point's
 //   Philox stream (counter (point, frame, draw / 4, 1); pair k = draws 2k,
 //   2k + 1 as 2u - 1; first k < 16 inside the disk, else the centre);
@@ -21,9 +21,9 @@
 // so the hit face, a decision, is reproducible.
 #include <cuda_runtime.h>
 
+#include "box_bins.cuh"
 #include "rll_device.cuh"
 #include "rll_internal.h"
-#include "sample_core.cuh"
 
 namespace rll {
 namespace {
@@ -37,12 +37,13 @@ constexpr float kPiF = 3.14159265358979323846f;
 __device__ __forceinline__ float fdivr(float a, float b) { return __fdiv_rn(a, b); }
 
 __global__ void __launch_bounds__(kBounceThreads)
-k_bounce(const float* __restrict__ pos, const float* __restrict__ nrm, int64_t np, const float* __restrict__ boxes,
+k_bounce(const float* __restrict__ pos, const float* __restrict__ nrm, int64_t np, const void* __restrict__ table,
          int n_boxes, float r0, float r1, float r2, float r3, float r4, float r5, uint2 key, uint32_t frame,
          float paths_per_tile, float* __restrict__ y_out, float* __restrict__ ny_out, float* __restrict__ fp_out)
 {
-    extern __shared__ float4 s_box[];
-    stage_boxes(s_box, boxes, n_boxes);
+    pdl_begin();
+    extern __shared__ float4 s_boxes[];
+    const BoxTable bt = stage_box_table(s_boxes, table, n_boxes);
     __syncthreads();
     const int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (p >= np) return;
@@ -95,8 +96,18 @@ k_bounce(const float* __restrict__ pos, const float* __restrict__ nrm, int64_t n
             axis = k;
         }
     }
-    // the nearest box face in front of it
-    for (int i = 0; i < n_boxes; ++i) {
+    // The nearest box face in front of it. A box whose face is met at t < t_best meets the segment's
+    // bounding box from o to there; widened by a margin above the rounding errors of the slab planes
+    // and of the segment's end (a few ulps of the coordinates), it keeps every box that counts.
+    float lo[3], hi[3];
+    for (int k = 0; k < 3; ++k) {
+        const float end = fadd(o[k], fmul(t_best, d[k]));  // NaN (every box kept) if d = 0 and no wall is ahead
+        const float e = 1e-5f * (1.0f + fabsf(o[k]) + fabsf(end));
+        lo[k] = fsub(end < o[k] ? end : o[k], e);
+        hi[k] = fadd(end > o[k] ? end : o[k], e);
+    }
+    const float4* s_box = bt.boxes();
+    bt.any(lo[0], lo[1], lo[2], hi[0], hi[1], hi[2], [&](int i) {
         const float4 lo4 = s_box[2 * i], hi4 = s_box[2 * i + 1];
         const float blo[3] = {lo4.x, lo4.y, lo4.z}, bhi[3] = {hi4.x, hi4.y, hi4.z};
         float tn = -INFINITY, tf = INFINITY;
@@ -120,7 +131,8 @@ k_bounce(const float* __restrict__ pos, const float* __restrict__ nrm, int64_t n
             t_best = tn;
             axis = ax;
         }
-    }
+        return false;
+    });
     if (t_best == INFINITY) {  // nothing ahead: the path escapes
         for (int k = 0; k < 3; ++k) {
             y_out[k * np + p] = o[k];
@@ -158,10 +170,15 @@ extern "C" int rll_bounce_vertices(rll_ctx* ctx, const float* pos, const float* 
         return fail(ctx, RLL_E_INVALID, "NULL point or output array");
     if (n_points == 0) return RLL_OK;
     DeviceGuard g(ctx->device);
+    const void* table = nullptr;
+    const int rc = box_table(ctx, boxes, n_boxes, ctx->stream, &table);
+    if (rc != RLL_OK) return rc;
     const unsigned blocks = (unsigned)((n_points + kBounceThreads - 1) / kBounceThreads);
-    const size_t smem = sizeof(float4) * 2 * (size_t)(n_boxes > 0 ? n_boxes : 1);
-    k_bounce<<<blocks, kBounceThreads, smem, ctx->stream>>>(
-        pos, nrm, n_points, boxes, n_boxes, room[0], room[1], room[2], room[3], room[4], room[5],
-        make_uint2((uint32_t)seed, (uint32_t)(seed >> 32)), frame, paths_per_tile, out_pos, out_nrm, out_footprint);
-    return check_cuda(ctx, cudaGetLastError(), "bounce kernel");
+    const size_t smem = n_boxes ? box_table_bytes(n_boxes) : 0;
+    return check_cuda(ctx,
+                      launch_pdl(k_bounce, dim3(blocks), dim3(kBounceThreads), smem, ctx->stream, pos, nrm, n_points,
+                                 table, (int)n_boxes, room[0], room[1], room[2], room[3], room[4], room[5],
+                                 make_uint2((uint32_t)seed, (uint32_t)(seed >> 32)), frame, paths_per_tile, out_pos,
+                                 out_nrm, out_footprint),
+                      "bounce kernel");
 }

@@ -9,8 +9,7 @@
 //   children per level, both bounds in packed f32x2 arithmetic) or a uniform
 //   pick over the cluster's lights
 //   uniform point on the light triangle, contribution, shadow segment vs the
-//   boxes (sorted by min.x once per call; only the run that can meet the
-//   segment is tested)
+//   boxes that can meet it (box_bins.cuh)
 //   estimate accumulation and one learning record (key, |c|).
 // The decisions (cell, branch, visibility) are exact binary32 formulas; the
 // cdf and descent comparisons u * total < c are made exactly with one fma.
@@ -40,27 +39,26 @@ template <int P, int MODE, bool DBG, int SPLIT, int THREADS, int MINB>
 __global__ void __launch_bounds__(THREADS, MINB) k_sample(SampleArgs a)
 {
     pdl_begin();
-    extern __shared__ float4 s_box[];
-    if (a.boxes_sorted) stage_sorted_boxes(s_box, a.boxes_sorted, a.n_boxes);
-    else stage_boxes(s_box, a.boxes, a.n_boxes);
+    extern __shared__ float4 s_boxes[];
+    const BoxTable bt = stage_box_table(s_boxes, a.box_table, a.n_boxes);
     if constexpr (SPLIT == LANES) {
         __shared__ float s_est[THREADS / 32][kWarpEst];
         __syncthreads();
         const uint32_t warp = threadIdx.x >> 5;
         const int64_t p0 = a.p_begin + ((int64_t)blockIdx.x * (THREADS / 32) + warp) * a.warp_points;
         if (p0 < a.p_end)
-            sample_points<P, MODE, DBG>(a, p0, (uint32_t)min((int64_t)a.warp_points, a.p_end - p0), s_box, s_est[warp]);
+            sample_points<P, MODE, DBG>(a, p0, (uint32_t)min((int64_t)a.warp_points, a.p_end - p0), bt, s_est[warp]);
     } else {
         __syncthreads();
         const int64_t p = a.p_begin + (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
         if (p >= a.p_end) return;
         if constexpr (SPLIT == ONE) {
             float est[3];
-            sample_one<P, MODE, DBG>(a, load_point(a, p), (uint32_t)p, s_box, est);
+            sample_one<P, MODE, DBG>(a, load_point(a, p), (uint32_t)p, bt, est);
 #pragma unroll
             for (int k = 0; k < 3; ++k) a.rgb[k * a.n_points + p] = est[k];
         } else {
-            sample_point<P, MODE, DBG>(a, p, s_box);
+            sample_point<P, MODE, DBG>(a, p, bt);
         }
     }
 }
@@ -68,8 +66,9 @@ __global__ void __launch_bounds__(THREADS, MINB) k_sample(SampleArgs a)
 // Energy-based baseline (Section 4): inversion of the cdf of leaf power.
 __global__ void __launch_bounds__(kThreads) k_sample_power(SampleArgs a, int32_t* light_out)
 {
-    extern __shared__ float4 s_box[];
-    stage_boxes(s_box, a.boxes, a.n_boxes);
+    pdl_begin();
+    extern __shared__ float4 s_boxes[];
+    const BoxTable bt = stage_box_table(s_boxes, a.box_table, a.n_boxes);
     __syncthreads();
     const int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (p >= a.n_points) return;
@@ -94,7 +93,7 @@ __global__ void __launch_bounds__(kThreads) k_sample_power(SampleArgs a, int32_t
         const float pl = a.nodes[nl - 1 + lo].phi / total;
         const LightRec Lr = load_light(a.lights + lo);
         const ShadeOut o = shade(Lr, x0, x1, x2, n0, n1, n2, alb, pl, 1.0f, rs.draw(kDrawTriA), rs.draw(kDrawTriB),
-                                 s_box, a.n_boxes, 0);
+                                 bt, 0);
         acc0 += o.est[0];
         acc1 += o.est[1];
         acc2 += o.est[2];
@@ -106,14 +105,11 @@ __global__ void __launch_bounds__(kThreads) k_sample_power(SampleArgs a, int32_t
     a.rgb[2 * np + p] = acc2 * inv_spp;
 }
 
-// The occluder boxes sorted for the shadow test (sort_boxes_block in sample_core.cuh), one block.
-constexpr int kSortBoxThreads = 256;
-
-__global__ void __launch_bounds__(kSortBoxThreads) k_sort_boxes(const float* __restrict__ boxes, int n,
-                                                                float4* __restrict__ out)
+// The table of the occluder boxes (box_bins.cuh), one block.
+__global__ void __launch_bounds__(256) k_box_table(const float* __restrict__ boxes, int n, char* __restrict__ out)
 {
     pdl_begin();
-    sort_boxes_block(boxes, n, out);
+    build_box_table(boxes, n, out);
 }
 
 template <int P, int MODE, bool DBG, int SPLIT, int THREADS, int MINB>
@@ -121,7 +117,7 @@ cudaError_t launch(const SampleArgs& a, cudaStream_t s)
 {
     const int64_t per_block = SPLIT == LANES ? (int64_t)(THREADS / 32) * a.warp_points : THREADS;
     const unsigned blocks = (unsigned)((a.p_end - a.p_begin + per_block - 1) / per_block);
-    const size_t smem = sizeof(float4) * 2 * (size_t)a.n_boxes;
+    const size_t smem = a.n_boxes ? box_table_bytes(a.n_boxes) : 0;
     return launch_pdl(k_sample<P, MODE, DBG, SPLIT, THREADS, MINB>, dim3(blocks), dim3(THREADS), smem, s, a);
 }
 
@@ -151,29 +147,29 @@ int sample_and_shade(rll_ctx* ctx, rll_grid* g, const rll_tree* t, const float* 
                      uint32_t frame, int spp, float* rgb, uint32_t* rec_key, float* rec_val,
                      const rll_sample_debug* dbg)
 {
-    const void* sorted = nullptr;
-    const int rc = sort_boxes(ctx, boxes, n_boxes, ctx->stream, &sorted);
+    const void* table = nullptr;
+    const int rc = box_table(ctx, boxes, n_boxes, ctx->stream, &table);
     if (rc != RLL_OK) return rc;
     return sample_and_shade_range(ctx, g, t, pos, nrm, albedo, footprint, n_points, 0, n_points, boxes, n_boxes, seed,
-                                  frame, spp, rgb, rec_key, rec_val, dbg, ctx->stream, sorted);
+                                  frame, spp, rgb, rec_key, rec_val, dbg, ctx->stream, table);
 }
 
-int sort_boxes(rll_ctx* ctx, const float* boxes, int n_boxes, cudaStream_t stream, const void** out)
+int box_table(rll_ctx* ctx, const float* boxes, int n_boxes, cudaStream_t stream, const void** out)
 {
     *out = nullptr;
     if (n_boxes <= 0) return RLL_OK;
-    if (!ctx->box_sorted) {
-        if (cudaMalloc(&ctx->box_sorted, sizeof(float4) * 2 * (size_t)kMaxBoxes) != cudaSuccess) {
+    if (!ctx->box_table) {
+        if (cudaMalloc(&ctx->box_table, kMaxBoxTable) != cudaSuccess) {
             cudaGetLastError();
-            ctx->box_sorted = nullptr;
-            return fail(ctx, RLL_E_NOMEM, "cannot allocate the sorted boxes");
+            ctx->box_table = nullptr;
+            return fail(ctx, RLL_E_NOMEM, "cannot allocate the box table");
         }
     }
     const int rc = check_cuda(ctx,
-                              launch_pdl(k_sort_boxes, dim3(1), dim3(kSortBoxThreads), 0, stream, boxes, n_boxes,
-                                         static_cast<float4*>(ctx->box_sorted)),
-                              "sort boxes");
-    if (rc == RLL_OK) *out = ctx->box_sorted;
+                              launch_pdl(k_box_table, dim3(1), dim3(256), 0, stream, boxes, n_boxes,
+                                         static_cast<char*>(ctx->box_table)),
+                              "box table");
+    if (rc == RLL_OK) *out = ctx->box_table;
     return rc;
 }
 
@@ -181,11 +177,11 @@ int sample_and_shade_range(rll_ctx* ctx, rll_grid* g, const rll_tree* t, const f
                            const float* albedo, const float* footprint, int64_t n_points, int64_t p_begin,
                            int64_t p_end, const float* boxes, int n_boxes, uint64_t seed, uint32_t frame, int spp,
                            float* rgb, uint32_t* rec_key, float* rec_val, const rll_sample_debug* dbg,
-                           cudaStream_t stream, const void* sorted_boxes)
+                           cudaStream_t stream, const void* table)
 {
     if (p_end <= p_begin) return RLL_OK;
     SampleArgs a{};
-    a.boxes_sorted = static_cast<const float4*>(sorted_boxes);
+    a.box_table = table;
     a.pos = pos;
     a.nrm = nrm;
     a.albedo = albedo;
@@ -247,6 +243,8 @@ int sample_power(rll_ctx* ctx, const rll_tree* t, const float* pos, const float*
 {
     if (n_points == 0) return RLL_OK;
     SampleArgs a{};
+    const int rc = box_table(ctx, boxes, n_boxes, ctx->stream, &a.box_table);
+    if (rc != RLL_OK) return rc;
     a.pos = pos;
     a.nrm = nrm;
     a.albedo = albedo;
@@ -262,8 +260,9 @@ int sample_power(rll_ctx* ctx, const rll_tree* t, const float* pos, const float*
     a.spp = spp;
     a.rgb = rgb;
     const unsigned blocks = (unsigned)((n_points + kThreads - 1) / kThreads);
-    k_sample_power<<<blocks, kThreads, sizeof(float4) * 2 * n_boxes, ctx->stream>>>(a, light_out);
-    return check_cuda(ctx, cudaGetLastError(), "sample_power");
+    const size_t smem = n_boxes ? box_table_bytes(n_boxes) : 0;
+    return check_cuda(ctx, launch_pdl(k_sample_power, dim3(blocks), dim3(kThreads), smem, ctx->stream, a, light_out),
+                      "sample_power");
 }
 
 }  // namespace rll

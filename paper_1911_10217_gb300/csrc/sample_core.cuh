@@ -6,7 +6,7 @@
 
 #include <cuda_runtime.h>
 
-#include "learn_core.cuh"  // bitonic_sort_u64
+#include "box_bins.cuh"
 #include "rll_device.cuh"
 
 namespace rll {
@@ -22,9 +22,7 @@ struct SampleArgs {
     int64_t p_begin, p_end;   // points this launch shades (k_sample)
     const float* boxes;
     int n_boxes;
-    // the boxes sorted by their lower x bound ([2 n_boxes] float4 (min, max); min.w the running
-    // maximum of max.x); nullptr: the boxes as given, all tested
-    const float4* boxes_sorted;
+    const void* box_table;    // of those boxes (box_bins.cuh; n_boxes > 0)
     unsigned long long* keys;
     const uint32_t* cut;
     const void* C;
@@ -126,13 +124,10 @@ struct ShadeOut {
     float reward;
 };
 
-// light point, shadow test, contribution (x, n: shading point and normal). s_box: the boxes,
-// s_box[2b] min and s_box[2b + 1] max; when `sorted`, in increasing order of min.x, with
-// s_box[2b].w the largest max.x among boxes 0..b.
+// light point, shadow test, contribution (x, n: shading point and normal)
 __device__ __forceinline__ ShadeOut shade(const LightRec& L, float x0, float x1, float x2, float n0, float n1,
                                           float n2, float albedo, float p_cut, float p_in, float ua, float ub,
-                                          const float4* s_box, int n_boxes, uint32_t reward_mode,
-                                          bool sorted = false)
+                                          const BoxTable& bt, uint32_t reward_mode)
 {
     const float su = fsqrt(ua);
     const float b0 = fsub(1.0f, su), b1 = fmul(ub, su), b2 = fsub(su, b1);
@@ -152,29 +147,10 @@ __device__ __forceinline__ ShadeOut shade(const LightRec& L, float x0, float x1,
     const float e0 = 1e-5f * (1.0f + fabsf(o0) + fabsf(y0));
     const float e1 = 1e-5f * (1.0f + fabsf(o1) + fabsf(y1));
     const float e2 = 1e-5f * (1.0f + fabsf(o2) + fabsf(y2));
-    const float lo0 = fminf(o0, y0) - e0, hi0 = fmaxf(o0, y0) + e0;
-    const float lo1 = fminf(o1, y1) - e1, hi1 = fmaxf(o1, y1) + e1;
-    const float lo2 = fminf(o2, y2) - e2, hi2 = fmaxf(o2, y2) + e2;
-    // With the boxes sorted by min.x, the boxes before the first one whose running maximum of max.x
-    // reaches lo0 all have max.x < lo0, and those from the first one with min.x > hi0 on all have
-    // min.x > hi0: the prefilter below rejects every box outside that run, so testing the run
-    // alone gives the decision of the full loop.
-    int b = 0;
-    const int b_end = n_boxes;
-    if (sorted) {
-        int lo = 0, hi = n_boxes;  // first box whose running maximum of max.x is >= lo0
-        while (lo < hi) {
-            const int mid = (lo + hi) >> 1;
-            if (s_box[2 * mid].w < lo0) lo = mid + 1;
-            else hi = mid;
-        }
-        b = lo;
-    }
-    bool occluded = false;
-    for (; b < b_end && !occluded; ++b) {
+    const float4* s_box = bt.boxes();
+    const bool occluded = bt.any(fminf(o0, y0) - e0, fminf(o1, y1) - e1, fminf(o2, y2) - e2, fmaxf(o0, y0) + e0,
+                                 fmaxf(o1, y1) + e1, fmaxf(o2, y2) + e2, [&](int b) {
         const float4 bmin = s_box[2 * b], bmax = s_box[2 * b + 1];
-        if (sorted && bmin.x > hi0) break;
-        if (bmin.x > hi0 || bmax.x < lo0 || bmin.y > hi1 || bmax.y < lo1 || bmin.z > hi2 || bmax.z < lo2) continue;
         const float ta0 = __fmaf_rn(bmin.x, i0, q0), tb0 = __fmaf_rn(bmax.x, i0, q0);
         const float ta1 = __fmaf_rn(bmin.y, i1, q1), tb1 = __fmaf_rn(bmax.y, i1, q1);
         const float ta2 = __fmaf_rn(bmin.z, i2, q2), tb2 = __fmaf_rn(bmax.z, i2, q2);
@@ -184,8 +160,8 @@ __device__ __forceinline__ ShadeOut shade(const LightRec& L, float x0, float x1,
         tf = fminf(tf, fmaxf(ta1, tb1));
         tn = fmaxf(tn, fminf(ta2, tb2));
         tf = fminf(tf, fmaxf(ta2, tb2));
-        occluded = tn < tf;
-    }
+        return tn < tf;
+    });
     ShadeOut o;
     const float wx = y0 - x0, wy = y1 - x1, wz = y2 - x2;
     const float d2 = wx * wx + wy * wy + wz * wz;
@@ -204,69 +180,6 @@ __device__ __forceinline__ ShadeOut shade(const LightRec& L, float x0, float x1,
     const float lum = 0.2126f * c0 + 0.7152f * c1 + 0.0722f * c2;
     o.reward = !(lum > 0.0f) ? 0.0f : (reward_mode == RLL_REWARD_CLUSTER ? __fdividef(lum * L.area, p_in) : lum * L.area);
     return o;
-}
-
-// MINB: resident blocks per SM the register allocation is held to (3: no
-// cap at 256 threads, 4: at most 64 registers per thread).
-// Boxes in shared memory as float4 pairs: s_box[2b] = (min xyz, 0),
-// s_box[2b + 1] = (max xyz, 0). Filled by all threads of the block.
-__device__ __forceinline__ void stage_boxes(float4* s_box, const float* boxes, int n_boxes)
-{
-    for (int b = threadIdx.x; b < n_boxes; b += blockDim.x) {
-        const float* bx = boxes + 6 * b;
-        s_box[2 * b] = make_float4(bx[0], bx[1], bx[2], 0.0f);
-        s_box[2 * b + 1] = make_float4(bx[3], bx[4], bx[5], 0.0f);
-    }
-}
-
-// The occluder boxes sorted by their lower x bound (ties by index) for the shadow test's early
-// start and stop, by the whole block: a bitonic network over (ordered min.x << 32 | index) keys in
-// shared memory. Output: [2 n] float4 (min, max) in that order, the min's w holding the running
-// maximum of max.x over the boxes up to this one (nondecreasing). n <= kMaxBoxes.
-struct SortBoxBarrier {
-    __device__ __forceinline__ void operator()() const { __syncthreads(); }
-};
-
-__device__ __forceinline__ void sort_boxes_block(const float* __restrict__ boxes, int n, float4* __restrict__ out)
-{
-    __shared__ unsigned long long s_key[kMaxBoxes];
-    __shared__ float s_hx[kMaxBoxes];  // max.x in sorted order, then its running maximum
-    for (int b = threadIdx.x; b < n; b += blockDim.x)
-        s_key[b] = ((unsigned long long)(uint32_t)(float_to_ordered(boxes[6 * b]) ^ (int)0x80000000) << 32) |
-                   (uint32_t)b;
-    __syncthreads();
-    bitonic_sort_u64(s_key, (uint32_t)n, threadIdx.x, blockDim.x, SortBoxBarrier{});
-    for (int i = threadIdx.x; i < n; i += blockDim.x) s_hx[i] = boxes[6 * (uint32_t)s_key[i] + 3];
-    __syncthreads();
-    if (threadIdx.x < 32) {  // running maximum: each lane scans a run, the lanes combine by shuffles
-        const int lane = threadIdx.x, per = (n + 31) / 32, b0 = lane * per, b1 = min(n, b0 + per);
-        float m = -INFINITY;
-        for (int i = b0; i < b1; ++i) m = fmaxf(m, s_hx[i]);
-        float incl = m;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const float y = __shfl_up_sync(0xffffffffu, incl, o);
-            if (lane >= o) incl = fmaxf(incl, y);
-        }
-        float run = __shfl_up_sync(0xffffffffu, incl, 1);
-        if (lane == 0) run = -INFINITY;
-        for (int i = b0; i < b1; ++i) {
-            run = fmaxf(run, s_hx[i]);
-            s_hx[i] = run;
-        }
-    }
-    __syncthreads();
-    for (int i = threadIdx.x; i < n; i += blockDim.x) {
-        const float* bx = boxes + 6 * (uint32_t)s_key[i];
-        out[2 * i] = make_float4(bx[0], bx[1], bx[2], s_hx[i]);
-        out[2 * i + 1] = make_float4(bx[3], bx[4], bx[5], 0.0f);
-    }
-}
-
-// The boxes as sorted by sort_boxes_block (2 n_boxes float4), copied as they are.
-__device__ __forceinline__ void stage_sorted_boxes(float4* s_box, const float4* sorted, int n_boxes)
-{
-    for (int i = threadIdx.x; i < 2 * n_boxes; i += blockDim.x) s_box[i] = sorted[i];
 }
 
 // Cell, cluster and triangle draws of one sample (draws 0-2 and 4-8).
@@ -459,10 +372,10 @@ __device__ __forceinline__ Point load_point(const SampleArgs& a, int64_t p)
                  a.footprint ? footprint_level(__ldg(a.footprint + p), a.h, a.levels) : 0u};
 }
 
-// Sample `sid` of a shading point, one thread (s_box: see stage_boxes): its estimate in est, its
-// learning record and diagnostics to their arrays.
+// Sample `sid` of a shading point, one thread: its estimate in est, its learning record and
+// diagnostics to their arrays.
 template <int P, int MODE, bool DBG>
-__device__ __forceinline__ void sample_one(const SampleArgs& a, const Point& pt, uint32_t sid, const float4* s_box,
+__device__ __forceinline__ void sample_one(const SampleArgs& a, const Point& pt, uint32_t sid, const BoxTable& bt,
                                            float est[3])
 {
     const float x0 = pt.x0, x1 = pt.x1, x2 = pt.x2, n0 = pt.n0, n1 = pt.n1, n2 = pt.n2, alb = pt.alb;
@@ -505,8 +418,7 @@ __device__ __forceinline__ void sample_one(const SampleArgs& a, const Point& pt,
         light = leaf_or_flag(a, node, nl1);
     }
     const LightRec Lr = load_light(a.lights + light);
-    const ShadeOut o = shade(Lr, x0, x1, x2, n0, n1, n2, alb, su.p_cut, p_in, su.ua, su.ub, s_box, a.n_boxes,
-                             a.reward_mode, a.boxes_sorted != nullptr);
+    const ShadeOut o = shade(Lr, x0, x1, x2, n0, n1, n2, alb, su.p_cut, p_in, su.ua, su.ub, bt, a.reward_mode);
     est[0] = o.est[0];
     est[1] = o.est[1];
     est[2] = o.est[2];
@@ -523,14 +435,14 @@ __device__ __forceinline__ void sample_one(const SampleArgs& a, const Point& pt,
 
 // All samples of shading point p, one thread.
 template <int P, int MODE, bool DBG>
-__device__ __forceinline__ void sample_point(const SampleArgs& a, int64_t p, const float4* s_box)
+__device__ __forceinline__ void sample_point(const SampleArgs& a, int64_t p, const BoxTable& bt)
 {
     const int64_t np = a.n_points;
     const Point pt = load_point(a, p);
     float acc[3] = {0.0f, 0.0f, 0.0f};
     for (int j = 0; j < a.spp; ++j) {
         float est[3];
-        sample_one<P, MODE, DBG>(a, pt, (uint32_t)(p * a.spp + j), s_box, est);
+        sample_one<P, MODE, DBG>(a, pt, (uint32_t)(p * a.spp + j), bt, est);
 #pragma unroll
         for (int k = 0; k < 3; ++k) acc[k] += est[k];
     }
@@ -578,7 +490,7 @@ inline uint32_t lane_split(int64_t n_points, int spp, int64_t warps)
 // (Whole passes: 200 x 120 points at 64 samples, 256-leaf cuts, 1 010 -> 458 us: a thread a point put
 // 1.2 blocks on an SM; 64 x 64 points at 4 samples 59 -> 48 us.)
 template <int P, int MODE, bool DBG>
-__device__ __forceinline__ void sample_points(const SampleArgs& a, int64_t p0, uint32_t count, const float4* s_box,
+__device__ __forceinline__ void sample_points(const SampleArgs& a, int64_t p0, uint32_t count, const BoxTable& bt,
                                               float* s_est)
 {
     const int64_t np = a.n_points;
@@ -588,7 +500,7 @@ __device__ __forceinline__ void sample_points(const SampleArgs& a, int64_t p0, u
     for (uint32_t base = 0; base < total; base += 32) {
         const uint32_t i = base + lane;
         float est[3] = {0.0f, 0.0f, 0.0f};
-        if (i < total) sample_one<P, MODE, DBG>(a, load_point(a, p0 + i / spp), (uint32_t)(p0 * a.spp) + i, s_box, est);
+        if (i < total) sample_one<P, MODE, DBG>(a, load_point(a, p0 + i / spp), (uint32_t)(p0 * a.spp) + i, bt, est);
 #pragma unroll
         for (int k = 0; k < 3; ++k) s_est[32 * k + lane] = est[k];
         __syncwarp();

@@ -1,0 +1,52 @@
+"""The occluder boxes' table (bins and masks) against the oracle, which tests
+every box: box counts at the table's steps (64-box words, bins halved above
+256), boxes of all sizes, flat ones, one that stretches the bins over a far
+larger extent (marked gpu)."""
+import dataclasses
+
+import numpy as np
+import pytest
+
+from paper_1911_10217_gb300 import scenes
+
+from .test_gpu_descent import check, env  # noqa: F401
+
+pytestmark = pytest.mark.gpu
+
+
+def random_boxes(n, far=False):
+    rng = np.random.default_rng(n)
+    size = np.exp(rng.uniform(np.log(2e-3), np.log(0.15), (n, 3)))
+    lo = rng.uniform(-0.1, 1.0, (n, 3))
+    hi = lo + size
+    hi[:: 7, 1] = lo[:: 7, 1]  # flat: never blocks
+    if far:
+        lo[0], hi[0] = (-1e4, 2.0, -1e4), (1e4, 3.0, 1e4)
+    return np.concatenate([lo, hi], axis=1).astype(np.float32)
+
+
+@pytest.mark.parametrize("n,far", [(1, False), (2, False), (63, False), (64, True), (65, False), (256, False),
+                                   (257, True), (1024, False)])
+def test_shadow_test_over_the_table(env, n, far):  # noqa: F811
+    s = dataclasses.replace(scenes.tiny_scene(), boxes=random_boxes(n, far))
+    check(env, s, frames=1, spp=2)
+
+
+@pytest.mark.parametrize("n,far", [(1, False), (64, True), (257, False), (1024, False)])
+def test_bounce_over_the_table(env, n, far):  # noqa: F811
+    """Vertices bit for bit, from points inside the room and outside it (paths that escape)."""
+    import torch
+    O, rll, ctx, dev = env["O"], env["rll"], env["ctx"], env["dev"]
+    boxes = random_boxes(n, far)
+    rng = np.random.default_rng(5)
+    P = 3001
+    pos = rng.uniform(-0.3, 1.3, (3, P)).astype(np.float32)
+    nrm = rng.normal(size=(3, P))
+    nrm[:, :64] = np.eye(3)[:, rng.integers(0, 3, 64)]
+    nrm = (nrm / np.linalg.norm(nrm, axis=0)).astype(np.float32)
+    oy, on, of = O.bounce_vertices(pos, nrm, boxes, scenes.ROOM, 9, 2, 50.0)
+    t = lambda a: torch.from_numpy(np.ascontiguousarray(a)).to(dev)  # noqa: E731
+    y, ny, f = torch.empty(3, P, device=dev), torch.empty(3, P, device=dev), torch.empty(P, device=dev)
+    rll.bounce_vertices(ctx, t(pos), t(nrm), t(boxes), scenes.ROOM, 9, 2, 50.0, y, ny, f)
+    for got, want in ((y, oy), (ny, on), (f, of)):
+        assert np.array_equal(got.cpu().numpy(), np.asarray(want, np.float32))
