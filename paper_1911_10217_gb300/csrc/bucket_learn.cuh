@@ -209,28 +209,35 @@ k_bucket_scatter(const uint32_t* __restrict__ rec_key, const float* __restrict__
     }
 }
 
-// Shared arrays of one team (a warp or a block) ordering one cell's records
-// (at most CAP records, cut sizes up to CLUS): A = bucket order, then
-// (cluster, sample) order; B = grouped by cluster, then the cdf scratch.
-template <uint32_t CAP, uint32_t CLUS = kMaxCut>
+// Shared arrays of one team (a warp, a pair of warps or a block) ordering one cell's records (at most
+// `cap` records, cut sizes up to CLUS), in the team's shared memory: A = bucket order, then (cluster,
+// sample) order; B = grouped by cluster.
+template <uint32_t CLUS>
 struct CellOrder {
-    uint32_t a_sid[CAP];
-    uint32_t a_val[CAP];
-    uint32_t b_sid[CAP];
-    uint32_t b_val[CAP];
-    uint8_t a_s[CAP];
-    uint8_t b_s[CAP];
-    uint32_t start[CLUS];  // first position of each cluster in B
-    uint32_t cur[CLUS];    // scatter cursors, then one past the last position
-    float q[CLUS];
-    // Once Eq. 1 is composed, the record arrays (the first 16 CAP bytes) are
-    // dead: they give the float and 16-bit scratch rows (CLUS entries each)
-    // of Eq. 2 and split-collapse.
-    static_assert(16u * CAP >= 6u * CLUS, "record arrays too small for the scratch rows");
-    __device__ __forceinline__ float* scratch_c() { return reinterpret_cast<float*>(this); }
-    __device__ __forceinline__ uint16_t* scratch_bits()
+    uint32_t *a_sid, *a_val, *b_sid, *b_val;
+    uint32_t *start;  // [CLUS] first position of each cluster in B
+    uint32_t *cur;    // [CLUS] scatter cursors, then one past the last position
+    float* q;         // [CLUS]
+    uint8_t *a_s, *b_s;
+    // Once Eq. 1 is composed, the record arrays (the first 16 cap bytes) are dead: they give the float
+    // and 16-bit scratch rows (CLUS entries each) of Eq. 2 and split-collapse.
+    float* scratch_c;
+    uint16_t* scratch_bits;
+
+    static constexpr size_t bytes(uint32_t cap) { return 18u * (size_t)cap + 12u * CLUS; }
+    __device__ __forceinline__ CellOrder(void* p, uint32_t cap)
     {
-        return reinterpret_cast<uint16_t*>(reinterpret_cast<char*>(this) + 4 * CLUS);
+        a_sid = static_cast<uint32_t*>(p);
+        a_val = a_sid + cap;
+        b_sid = a_val + cap;
+        b_val = b_sid + cap;
+        start = b_val + cap;
+        cur = start + CLUS;
+        q = reinterpret_cast<float*>(cur + CLUS);
+        a_s = reinterpret_cast<uint8_t*>(q + CLUS);
+        b_s = a_s + cap;
+        scratch_c = static_cast<float*>(p);
+        scratch_bits = reinterpret_cast<uint16_t*>(scratch_c + CLUS);
     }
 };
 
@@ -267,31 +274,25 @@ struct WithSplit {
 };
 
 
-// A team orders one cell; its first warp (lead()) also scans and composes.
-struct WarpTeam {
-    __device__ __forceinline__ uint32_t tid() const { return threadIdx.x & 31; }
-    __device__ __forceinline__ uint32_t size() const { return 32; }
-    __device__ __forceinline__ bool lead() const { return true; }
-    __device__ __forceinline__ void sync() const { __syncwarp(); }
-};
-struct BlockTeam {
-    __device__ __forceinline__ uint32_t tid() const { return threadIdx.x; }
-    __device__ __forceinline__ uint32_t size() const { return blockDim.x; }
-    __device__ __forceinline__ bool lead() const { return threadIdx.x < 32; }
-    __device__ __forceinline__ void sync() const { __syncthreads(); }
-};
-// warps 2p and 2p + 1 of a block; named barrier 1 + p (0 is __syncthreads)
-struct PairTeam {
-    __device__ __forceinline__ uint32_t tid() const { return threadIdx.x & 63u; }
-    __device__ __forceinline__ uint32_t size() const { return 64; }
-    __device__ __forceinline__ bool lead() const { return (threadIdx.x & 63u) < 32u; }
-    // immediate barrier ids (a register id would reserve all 16 barriers of the block)
+// The threads that order one cell together; its first warp also scans and finishes. One kind of object
+// for all three sizes, so that the learning kernel holds its per-cell code once (a copy for each size
+// was 3 % slower at 64x64 points and 1 % at 128 leaves, equal elsewhere; see warp_rebuild_cdf).
+struct Team {
+    uint32_t tid, size;  // 32, 64 or the block
+    __device__ __forceinline__ bool lead() const { return tid < 32; }
     __device__ __forceinline__ void sync() const
     {
-        switch (threadIdx.x >> 6) {
-        case 0: asm volatile("bar.sync 1, 64;" ::: "memory"); break;
-        case 1: asm volatile("bar.sync 2, 64;" ::: "memory"); break;
-        default: asm volatile("bar.sync 3, 64;" ::: "memory"); break;
+        if (size == 32) {
+            __syncwarp();
+        } else if (size == 64) {  // warps 2p and 2p + 1: named barrier 1 + p (0 is __syncthreads)
+            // immediate barrier ids (a register id would reserve all 16 barriers of the block)
+            switch (threadIdx.x >> 6) {
+            case 0: asm volatile("bar.sync 1, 64;" ::: "memory"); break;
+            case 1: asm volatile("bar.sync 2, 64;" ::: "memory"); break;
+            default: asm volatile("bar.sync 3, 64;" ::: "memory"); break;
+            }
+        } else {
+            __syncthreads();
         }
     }
 };
@@ -299,15 +300,17 @@ struct BlockSync {
     __device__ __forceinline__ void operator()() const { __syncthreads(); }
 };
 
-template <int P>
+template <int P, int U = 4>
 __device__ __forceinline__ void load_q_row(const typename Store<P>::T* qrow, uint32_t m, float* q)
 {
+#pragma unroll U
     for (uint32_t s = threadIdx.x & 31; s < m; s += 32) q[s] = Store<P>::load(qrow[s]);
 }
 
-template <int P>
+template <int P, int U = 4>
 __device__ __forceinline__ void store_q_row(typename Store<P>::T* qrow, uint32_t m, float* q)
 {
+#pragma unroll U
     for (uint32_t s = threadIdx.x & 31; s < m; s += 32) {
         const typename Store<P>::T st = Store<P>::store(q[s]);
         qrow[s] = st;
@@ -319,20 +322,21 @@ __device__ __forceinline__ void store_q_row(typename Store<P>::T* qrow, uint32_t
 // precision (q then holds the stored values); with a split policy,
 // split-collapse on those values and the rows it changed stored; then Eq. 2
 // from the final Q. Scratch rows of kMaxCut entries: cs, nc, c, bits.
-template <int P, class Split>
+template <int P, int U = 4, class Split>
 __device__ void finish_cell(const Split& sp, uint32_t slot, float* q, uint32_t m, float eps,
                             typename Store<P>::T* qrow, typename Store<P>::T* crow, uint32_t* cs, uint32_t* nc,
                             float* c, uint16_t* bits, uint32_t* status)
 {
-    store_q_row<P>(qrow, m, q);
+    store_q_row<P, U>(qrow, m, q);
     __syncwarp();
     if constexpr (Split::kOn) {
         const int lane = threadIdx.x & 31;
         const SplitRow r = sp.row(slot);
-        if (load_cut_row(r.cut, cs, m, r.n_nodes, status)) {
-            const uint32_t steps = split_collapse_steps<P>(cs, q, c, nc, m, r.nodes, r.parent, r.left, r.right, r.T,
-                                                           r.max_iter, r.n_nodes);
+        if (load_cut_row<U>(r.cut, cs, m, r.n_nodes, status)) {
+            const uint32_t steps = split_collapse_steps<P, U>(cs, q, c, nc, m, r.nodes, r.parent, r.left, r.right,
+                                                              r.T, r.max_iter, r.n_nodes);
             if (steps) {
+#pragma unroll U
                 for (uint32_t s = lane; s < m; s += 32) {
                     r.cut[s] = cs[s];
                     qrow[s] = Store<P>::store(q[s]);  // exact: q holds table values
@@ -341,24 +345,27 @@ __device__ void finish_cell(const Split& sp, uint32_t slot, float* q, uint32_t m
             }
         }
     }
-    warp_rebuild_cdf<P>(q, (int)m, eps, crow, c, bits);
+    warp_rebuild_cdf<P, U>(q, (int)m, eps, crow, c, bits);
 }
 
-// Eq. 1 + Eq. 2 of one cell from its bucket of nr <= CAP records: grouped
+// Eq. 1 + Eq. 2 of one cell from its bucket of nr <= cap records: grouped
 // by cluster (counting sort, any order inside a group), then each record's
 // rank by sample id inside its group is counted, which puts them in
 // (cluster, sample) order; warp 0 of the team composes, stores Q and
 // rebuilds C. Called by every thread of the team.
-template <int P, uint32_t CAP, uint32_t CLUS, class Team, class Split>
-__device__ void learn_cell_grouped(Team team, CellOrder<CAP, CLUS>& o, const Bucket& bucket, uint32_t b0, uint32_t nr,
-                                   uint32_t M, uint32_t m, float alpha, float eps, typename Store<P>::T* qrow,
-                                   typename Store<P>::T* crow, const Split& sp, uint32_t slot, uint32_t* status)
+template <int P, uint32_t CLUS, class Split>
+__device__ __forceinline__ void learn_cell_grouped(const Team& team, const CellOrder<CLUS>& o, const Bucket& bucket,
+                                                   uint32_t b0, uint32_t nr, uint32_t M, uint32_t m, float alpha,
+                                                   float eps, typename Store<P>::T* qrow, typename Store<P>::T* crow,
+                                                   const Split& sp, uint32_t slot, uint32_t* status)
 {
-    const uint32_t t = team.tid(), T = team.size();
+    constexpr int U = CLUS <= 64 ? 1 : 4;  // see warp_rebuild_cdf
+    const uint32_t t = team.tid, T = team.size;
     const int lane = threadIdx.x & 31;
     const bool w0 = team.lead();
+#pragma unroll U
     for (uint32_t s = t; s < M; s += T) o.start[s] = 0u;
-    if (w0) load_q_row<P>(qrow, m, o.q);
+    if (w0) load_q_row<P, U>(qrow, m, o.q);
     team.sync();
     // the bucket, four records a thread in flight at once
     for (uint32_t k0 = t; k0 < nr; k0 += 4 * T) {
@@ -384,6 +391,7 @@ __device__ void learn_cell_grouped(Team team, CellOrder<CAP, CLUS>& o, const Buc
     if (w0) {  // cluster starts: exclusive scan over M bins, ipl consecutive bins a lane
         const uint32_t ipl = (M + 31) >> 5, lo = lane * ipl, hi = min(M, lo + ipl);
         uint32_t sum = 0;
+#pragma unroll U
         for (uint32_t s = lo; s < hi; ++s) sum += o.start[s];
         uint32_t y = sum;
 #pragma unroll
@@ -392,6 +400,7 @@ __device__ void learn_cell_grouped(Team team, CellOrder<CAP, CLUS>& o, const Buc
             if (lane >= d) y += v;
         }
         uint32_t run = y - sum;
+#pragma unroll U
         for (uint32_t s = lo; s < hi; ++s) {
             const uint32_t c = o.start[s];
             o.start[s] = run;
@@ -434,6 +443,7 @@ __device__ void learn_cell_grouped(Team team, CellOrder<CAP, CLUS>& o, const Buc
         learn_records<P>([&](uint32_t j) { return make_uint2(o.a_s[j], o.a_val[j]); }, nr, m, alpha, o.q);
     } else {  // a block or a pair: warp w of the team composes the groups of clusters w, w + warps, ...
         const uint32_t warps = T >> 5;
+#pragma unroll U
         for (uint32_t s = t >> 5; s < M; s += warps) {
             const uint32_t lo = o.start[s], hi = o.cur[s];
             if (hi > lo)
@@ -443,7 +453,7 @@ __device__ void learn_cell_grouped(Team team, CellOrder<CAP, CLUS>& o, const Buc
         team.sync();
     }
     if (w0)  // cluster starts and cursors are dead too: the cut scratch rows
-        finish_cell<P>(sp, slot, o.q, m, eps, qrow, crow, o.start, o.cur, o.scratch_c(), o.scratch_bits(), status);
+        finish_cell<P, U>(sp, slot, o.q, m, eps, qrow, crow, o.start, o.cur, o.scratch_c, o.scratch_bits, status);
 }
 
 // Eq. 1 of one cell whose records are sorted by (cluster, sample id), by a
@@ -472,11 +482,11 @@ __device__ void compose_sorted_block(Cls cls, Val val, uint32_t nr, uint32_t M, 
 }
 
 // 4. Eq. 1 + Eq. 2 of every touched cell of at most kBlockGroup records in
-// one persistent launch. Phase 1: blocks take the cells of the block list
+// one persistent launch. Phase 0: blocks take the cells of the block list
 // (more than kPairBucket records; the ordering of the warp path done by the
-// whole block, warps composing different clusters in parallel). Phase 2: the
+// whole block, warps composing different clusters in parallel). Phase 1: the
 // block's warp pairs take the cells of the two-warp list (kWarpBucket ..
-// kPairBucket records), three cells per block at a time. Phase 3: warps take
+// kPairBucket records), three cells per block at a time. Phase 2: warps take
 // the touched cells one by one and order those of at most kWarpBucket records
 // themselves. Every phase draws from an atomic work counter (ctr[4], ctr[7],
 // ctr[5]), so the long cells start first and the teams that drew one join the
@@ -485,9 +495,11 @@ __device__ void compose_sorted_block(Cls cls, Val val, uint32_t nr, uint32_t M, 
 // a pair's arrays lie in its two warps' slabs, the block's across all.
 template <uint32_t CLUS>
 struct LearnSmem {
-    static constexpr size_t kWarp = sizeof(CellOrder<kWarpBucket, CLUS>);
-    static constexpr size_t kPairHalf = (sizeof(CellOrder<kPairBucket, CLUS>) + 1) / 2;
-    static constexpr size_t kSlab = ((kWarp > kPairHalf ? kWarp : kPairHalf) + 15) & ~(size_t)15;
+    using O = CellOrder<CLUS>;
+    static constexpr size_t kPairHalf = (O::bytes(kPairBucket) + 1) / 2;
+    static constexpr size_t kSlab = ((O::bytes(kWarpBucket) > kPairHalf ? O::bytes(kWarpBucket) : kPairHalf) + 15) &
+                                    ~(size_t)15;
+    static_assert(16u * kWarpBucket >= 6u * CLUS, "record arrays too small for the scratch rows");
 };
 
 template <int P, int WARPS, int MINB, uint32_t CLUS, class Rows, class Split>
@@ -500,66 +512,58 @@ k_learn_buckets(const Bucket bucket, uint32_t* __restrict__ ctr, const uint32_t*
     pdl_begin();
     static_assert(WARPS == 6, "three warp pairs, named barriers 1 .. 3");
     using L = LearnSmem<CLUS>;
-    static_assert(sizeof(CellOrder<kBlockGroup, CLUS>) <= WARPS * L::kSlab, "block arrays exceed the slabs");
+    static_assert(CellOrder<CLUS>::bytes(kBlockGroup) <= WARPS * L::kSlab, "block arrays exceed the slabs");
     __shared__ __align__(16) unsigned char smem[WARPS * L::kSlab];
     __shared__ uint32_t s_next, s_pair[WARPS / 2];
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const uint32_t warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const uint32_t n_group = *(volatile const uint32_t*)(ctr + 6);
     const uint32_t n_pair = *(volatile const uint32_t*)(ctr + 3);
     const uint32_t total = *(volatile const uint32_t*)ctr;
-    auto& block_order = *reinterpret_cast<CellOrder<kBlockGroup, CLUS>*>(smem);
+    uint32_t phase = n_group ? 0u : (n_pair ? 1u : 2u), ahead = 0;
+    bool drawn = false;  // phase 2: `ahead` holds the next index
     for (;;) {
-        if (threadIdx.x == 0) s_next = atomicAdd(ctr + 4, 1u);
-        __syncthreads();
-        const uint32_t bi = s_next;
-        __syncthreads();
-        if (bi >= n_group) break;  // uniform across the block
-        const uint32_t w = group_list[cells - 1u - bi];
-        const uint32_t slot = touched[w], b0 = start[w], nr = len[w];
+        uint32_t w;  // index of the next cell in the touched list
+        Team team;
+        if (phase == 0) {
+            if (threadIdx.x == 0) s_next = atomicAdd(ctr + 4, 1u);
+            __syncthreads();
+            const uint32_t bi = s_next;
+            __syncthreads();
+            if (bi >= n_group) {  // uniform across the block: every warp leaves phase 0
+                phase = 1;
+                continue;
+            }
+            w = group_list[cells - 1u - bi];
+            team = Team{threadIdx.x, (uint32_t)(WARPS * 32)};
+        } else if (phase == 1) {
+            team = Team{threadIdx.x & 63u, 64u};
+            if (team.tid == 0) s_pair[warp >> 1] = atomicAdd(ctr + 7, 1u);
+            team.sync();
+            const uint32_t pi = s_pair[warp >> 1];
+            team.sync();
+            if (pi >= n_pair) {  // uniform across the pair: the shared memory is per warp now
+                phase = 2;
+                continue;
+            }
+            w = group_list[pi];
+        } else {
+            team = Team{lane, 32u};
+            if (!drawn && lane == 0) ahead = atomicAdd(ctr + 5, 1u);
+            w = __shfl_sync(0xffffffffu, ahead, 0);
+            if (w >= total) break;
+            if (lane == 0) ahead = atomicAdd(ctr + 5, 1u);
+            drawn = true;
+        }
+        const uint32_t slot = touched[w], nr = len[w];
+        if (phase == 2 && nr > kWarpBucket) continue;
+        const uint32_t b0 = start[w];
         const RowRef<P> r = rows.row(slot);
-        learn_cell_grouped<P>(BlockTeam{}, block_order, bucket, b0, nr, r.M, r.m,
-                              r.alpha, r.eps, r.Q, r.C, sp, slot, status);
-        if (threadIdx.x == 0) cursor[slot] = 0u;
-        __syncthreads();
-    }
-    // every warp of the block has left phase 1: pairs of warps, each in its own two slabs
-    {
-        const PairTeam team;
-        const int pair = warp >> 1;
-        auto& pair_order = *reinterpret_cast<CellOrder<kPairBucket, CLUS>*>(smem + 2 * pair * L::kSlab);
-        for (;;) {
-            if (team.tid() == 0) s_pair[pair] = atomicAdd(ctr + 7, 1u);
-            team.sync();
-            const uint32_t pi = s_pair[pair];
-            team.sync();
-            if (pi >= n_pair) break;  // uniform across the pair
-            const uint32_t w = group_list[pi];
-            const uint32_t slot = touched[w], b0 = start[w], nr = len[w];
-            const RowRef<P> r = rows.row(slot);
-            learn_cell_grouped<P>(team, pair_order, bucket, b0, nr, r.M, r.m,
-                                  r.alpha, r.eps, r.Q, r.C, sp, slot, status);
-            if (team.tid() == 0) cursor[slot] = 0u;
-            team.sync();
-        }
-    }
-    // both warps of the pair have left phase 2: the shared memory is per warp now
-    auto& warp_order = *reinterpret_cast<CellOrder<kWarpBucket, CLUS>*>(smem + warp * L::kSlab);
-    uint32_t next = 0;
-    if (lane == 0) next = atomicAdd(ctr + 5, 1u);
-    next = __shfl_sync(0xffffffffu, next, 0);
-    while (next < total) {
-        const uint32_t i = next;
-        uint32_t ahead = 0;
-        if (lane == 0) ahead = atomicAdd(ctr + 5, 1u);
-        const uint32_t slot = touched[i], nr = len[i];
-        if (nr <= kWarpBucket) {
-            const RowRef<P> r = rows.row(slot);
-            const uint32_t b0 = start[i];
-            learn_cell_grouped<P>(WarpTeam{}, warp_order, bucket, b0, nr, r.M,
-                                  r.m, r.alpha, r.eps, r.Q, r.C, sp, slot, status);
-            if (lane == 0) cursor[slot] = 0u;
-        }
-        next = __shfl_sync(0xffffffffu, ahead, 0);
+        const uint32_t slab = phase == 0 ? 0u : (phase == 1 ? warp & ~1u : warp);
+        const uint32_t cap = phase == 0 ? kBlockGroup : (phase == 1 ? kPairBucket : kWarpBucket);
+        learn_cell_grouped<P>(team, CellOrder<CLUS>(smem + slab * L::kSlab, cap), bucket, b0, nr, r.M, r.m, r.alpha,
+                              r.eps, r.Q, r.C, sp, slot, status);
+        if (team.tid == 0) cursor[slot] = 0u;
+        if (phase != 2) team.sync();
     }
 }
 

@@ -18,15 +18,22 @@ __device__ __forceinline__ float warp_sum(float v)
     return v;
 }
 
+// U: how far the loops over a row's entries are unrolled (one entry a lane and turn): 1 for cuts of at
+// most 64 leaves, where a lane has one or two turns and unrolling only lengthens the code (the learning
+// kernel's warps, each at another place of it, waited for instructions a fifth of the time: 4K
+// bfloat16, 64 leaves, whole passes 1 975 -> 1 883 us, 1080p 418 -> 407), 4 for larger ones, whose
+// four to eight turns it overlaps (128 leaves: 645 us a pass against 655).
+
 // Eq. 2 with the floor: q holds the stored Q of one row (m values, shared
 // memory); c and bits are shared scratch of the same length. Writes the
 // stored cdf row. Called by all 32 lanes of a warp.
-template <int P>
+template <int P, int U = 4>
 __device__ void warp_rebuild_cdf(const float* q, int m, float eps, typename Store<P>::T* out, float* c,
                                  uint16_t* bits)
 {
     const int lane = threadIdx.x & 31;
     float part = 0.0f, qmax = 0.0f;
+#pragma unroll U
     for (int s = lane; s < m; s += 32) {
         part += q[s];
         qmax = fmaxf(qmax, q[s]);
@@ -40,6 +47,7 @@ __device__ void warp_rebuild_cdf(const float* q, int m, float eps, typename Stor
     const int ipl = (m + 31) >> 5;
     const int b = lane * ipl, e = min(m, b + ipl);
     float run = 0.0f;
+#pragma unroll U
     for (int s = b; s < e; ++s) {
         run += uniform ? 1.0f : q[s] + add;
         c[s] = run;
@@ -51,14 +59,17 @@ __device__ void warp_rebuild_cdf(const float* q, int m, float eps, typename Stor
         if (lane >= o) x += y;
     }
     const float before = x - run;
+#pragma unroll U
     for (int s = b; s < e; ++s) c[s] += before;
     __syncwarp();
     if constexpr (P == RLL_PREC_FP32) {
+#pragma unroll U
         for (int s = lane; s < m; s += 32) out[s] = Store<P>::store(c[s]);
         __syncwarp();
         return;
     } else {
         const float total = c[m - 1];
+#pragma unroll U
         for (int s = lane; s < m; s += 32) bits[s] = Store<P>::bits(Store<P>::store(c[s] / total));
         __syncwarp();
         // Strictly increasing bit patterns (positive values order as their bits), last = 1.0:
@@ -114,6 +125,7 @@ __device__ void warp_rebuild_cdf(const float* q, int m, float eps, typename Stor
             }
         }
         __syncwarp();
+#pragma unroll U
         for (int s = lane; s < m; s += 32) out[s] = Store<P>::from_bits(bits[s]);
         __syncwarp();
     }
@@ -257,6 +269,7 @@ __device__ void learn_records(Get get, uint32_t len, uint32_t m, float alpha, fl
 {
     const int lane = threadIdx.x & 31;
     const float a1 = 1.0f - alpha;
+#pragma unroll 1
     for (uint32_t pos = 0; pos < len; pos += 32) {
         const uint32_t j = pos + lane;
         const bool valid = j < len;
@@ -287,7 +300,7 @@ __device__ void learn_records(Get get, uint32_t len, uint32_t m, float alpha, fl
 // New Q values in correctly rounded binary32, then rounded to the table
 // precision: l_max's Q times f = phi_a / (phi_a + phi_c) and times 1 - f
 // (children's power), p_min's Q the sum of its children's. One warp.
-template <int P>
+template <int P, int U = 4>
 __device__ uint32_t split_collapse_steps(uint32_t* cs, float* q, float* c, uint32_t* nc, uint32_t m,
                                 const NodeRec* __restrict__ nodes, const int32_t* __restrict__ parent,
                                 const int32_t* __restrict__ left, const int32_t* __restrict__ right, float T,
@@ -298,6 +311,7 @@ __device__ uint32_t split_collapse_steps(uint32_t* cs, float* q, float* c, uint3
     uint32_t steps = 0;
     for (; steps < max_iter; ++steps) {
         ArgBest hi{0.0f, 0xFFFFFFFFu}, lo{0.0f, 0xFFFFFFFFu};
+#pragma unroll U
         for (uint32_t s = lane; s < m; s += 32) {
             if (cs[s] < n_internal && (hi.i == 0xFFFFFFFFu || q[s] > hi.v)) {
                 hi.v = q[s];
@@ -329,6 +343,7 @@ __device__ uint32_t split_collapse_steps(uint32_t* cs, float* q, float* c, uint3
         const float sum = fadd(pa, pc);
         const float fa = sum > 0.0f ? fdiv(pa, sum) : 0.5f;
         float* nq = c;
+#pragma unroll U
         for (uint32_t i = lane; i < m; i += 32) {
             if (i == L + 1) continue;
             const uint32_t k = i + (i > H ? 1u : 0u) - (i > L + 1 ? 1u : 0u);
@@ -346,6 +361,7 @@ __device__ uint32_t split_collapse_steps(uint32_t* cs, float* q, float* c, uint3
             }
         }
         __syncwarp();
+#pragma unroll U
         for (uint32_t i = lane; i < m; i += 32) {
             cs[i] = nc[i];
             q[i] = nq[i];
@@ -357,11 +373,13 @@ __device__ uint32_t split_collapse_steps(uint32_t* cs, float* q, float* c, uint3
 
 // Loads cut row crow into cs (m entries); false (and RLL_E_DEVICE flagged)
 // when an entry is not a node of the tree. One warp.
+template <int U = 4>
 __device__ __forceinline__ bool load_cut_row(const uint32_t* crow, uint32_t* cs, uint32_t m, int64_t n_nodes,
                                              uint32_t* status)
 {
     const int lane = threadIdx.x & 31;
     bool bad = false;
+#pragma unroll U
     for (uint32_t s = lane; s < m; s += 32) {
         cs[s] = crow[s];
         bad |= (int64_t)cs[s] >= n_nodes;
