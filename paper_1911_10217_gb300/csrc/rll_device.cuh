@@ -336,6 +336,11 @@ __device__ __forceinline__ float2 neg_sqrt2(float2 n)
 // Fewer instructions than with the library's square root and scalar negations
 // (whole passes: 64x64 points 60.6 -> 58.1 us, 1080p 470.9 -> 463.5 us, 4K
 // bfloat16 2 224 -> 2 195 us; the record loads bound the kernel at that point).
+namespace {
+// out of line: the path of nodes out of neg_sqrt2's range, which is rarely taken, costs the descent
+// loop no code (see sample_one)
+__device__ __noinline__ float far_sqrt(float x) { return fsqrt(x); }
+}  // namespace
 struct Bound2 {
     float2 num, den;
 };
@@ -370,9 +375,9 @@ __device__ __forceinline__ Bound2 importance2(const NodePair& q, float2 phi, flo
         nsr = neg_sqrt2(xr);
         nse = neg_sqrt2(xe);
     } else {
-        ncb = make_float2(-fsqrt(-nt.x), -fsqrt(-nt.y));
-        nsr = make_float2(-fsqrt(-xr.x), -fsqrt(-xr.y));
-        nse = make_float2(-fsqrt(-xe.x), -fsqrt(-xe.y));
+        ncb = make_float2(-far_sqrt(-nt.x), -far_sqrt(-nt.y));
+        nsr = make_float2(-far_sqrt(-xr.x), -far_sqrt(-xr.y));
+        nse = make_float2(-far_sqrt(-xe.x), -far_sqrt(-xe.y));
     }
     float2 A = d2, B = d2;
     {
