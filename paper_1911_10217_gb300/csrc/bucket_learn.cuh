@@ -35,9 +35,12 @@ constexpr int kTilesPerWarp = 4;         // 32-record tiles one warp counts / sc
 constexpr uint32_t kWarpBucket = 240;    // records of a cell one warp orders in shared memory
 constexpr uint32_t kPairBucket = 512;    // records of a cell two warps order together
 constexpr uint32_t kBlockGroup = 1024;   // records of a cell one block orders by grouping and ranking
-constexpr uint32_t kBlockSort = 8192;    // records of a cell one block sorts in shared memory (power of 2)
-constexpr size_t kBigSmem = kBlockSort * (sizeof(unsigned long long) + sizeof(uint32_t));
-constexpr int kBigThreads = 512;
+constexpr int kBigThreads = 1024;
+constexpr uint32_t kBlockSort = 8 * kBigThreads;  // records of a cell one block sorts in shared memory, one tile
+constexpr uint32_t kDigits = 256;
+// two arrays of a tile's records, and the warps' digit counters (radix_pass)
+constexpr size_t kBigSmem =
+    2 * kBlockSort * sizeof(unsigned long long) + (kBigThreads / 32 + 1) * kDigits * sizeof(uint32_t);
 
 // 1. record counts per cell and each record's rank among its cell's records
 // (the cell's count before its warp's group, plus the lanes of the group
@@ -296,10 +299,6 @@ struct Team {
         }
     }
 };
-struct BlockSync {
-    __device__ __forceinline__ void operator()() const { __syncthreads(); }
-};
-
 template <int P, int U = 4>
 __device__ __forceinline__ void load_q_row(const typename Store<P>::T* qrow, uint32_t m, float* q)
 {
@@ -443,12 +442,13 @@ __device__ __forceinline__ void learn_cell_grouped(const Team& team, const CellO
         learn_records<P>([&](uint32_t j) { return make_uint2(o.a_s[j], o.a_val[j]); }, nr, m, alpha, o.q);
     } else {  // a block or a pair: warp w of the team composes the groups of clusters w, w + warps, ...
         const uint32_t warps = T >> 5;
+        const GroupScan scan(alpha);
 #pragma unroll U
         for (uint32_t s = t >> 5; s < M; s += warps) {
             const uint32_t lo = o.start[s], hi = o.cur[s];
-            if (hi > lo)
-                learn_records<P>([&](uint32_t j) { return make_uint2(o.a_s[lo + j], o.a_val[lo + j]); }, hi - lo,
-                                 m, alpha, o.q);
+            if (hi <= lo || s >= m) continue;
+            const float q = scan.run([&](uint32_t j) { return o.a_val[lo + j]; }, hi - lo, o.q[s]);
+            if (lane == 0) o.q[s] = q;
         }
         team.sync();
     }
@@ -474,9 +474,12 @@ __device__ void compose_sorted_block(Cls cls, Val val, uint32_t nr, uint32_t M, 
     }
     __syncthreads();
     const uint32_t warps = blockDim.x >> 5;
+    const GroupScan scan(alpha);
     for (uint32_t s = threadIdx.x >> 5; s < M; s += warps) {
         const uint32_t lo = gs[s], hi = ge[s];
-        if (hi > lo) learn_records<P>([&](uint32_t j) { return make_uint2(s, val(lo + j)); }, hi - lo, m, alpha, q);
+        if (hi <= lo || s >= m) continue;
+        const float qs = scan.run([&](uint32_t j) { return val(lo + j); }, hi - lo, q[s]);
+        if ((threadIdx.x & 31) == 0) q[s] = qs;
     }
     __syncthreads();
 }
@@ -509,7 +512,15 @@ k_learn_buckets(const Bucket bucket, uint32_t* __restrict__ ctr, const uint32_t*
                 const uint32_t* __restrict__ len, uint32_t* __restrict__ cursor, Rows rows, Split sp,
                 uint32_t* __restrict__ status, uint32_t cells)
 {
-    pdl_begin();
+    // Launched after k_learn_big, whose cells are others. Where it has cells, this kernel runs beside
+    // it: it starts when every block of k_learn_big has released it, that is when the scatter is
+    // complete and visible (each block waits for it first), and ends only when k_learn_big has, so
+    // that whatever follows this kernel follows both. Where it has none, k_learn_big releases this
+    // kernel at once and ends with the scatter, for which this kernel's blocks wait in their places.
+    // (The claim, which writes the counts, is complete before any block of the scatter releases.)
+    const bool beside = *(volatile const uint32_t*)(ctr + 2) != 0u;
+    if (!beside) pdl_wait();
+    pdl_release();
     static_assert(WARPS == 6, "three warp pairs, named barriers 1 .. 3");
     using L = LearnSmem<CLUS>;
     static_assert(CellOrder<CLUS>::bytes(kBlockGroup) <= WARPS * L::kSlab, "block arrays exceed the slabs");
@@ -565,28 +576,144 @@ k_learn_buckets(const Bucket bucket, uint32_t* __restrict__ ctr, const uint32_t*
         if (team.tid == 0) cursor[slot] = 0u;
         if (phase != 2) team.sync();
     }
+    if (beside) pdl_wait();
 }
 
-// 5b. one block per cell of the sorting list. Up to kBlockSort records: keys
-// cluster << 45 | sample id << 13 | bucket index sorted by a bitonic network
-// in shared memory, rewards gathered in that order. Larger cells: (cluster
-// << 32 | sample id) sorted in place in global scratch, rewards read by
-// sample id. Then Eq. 1 (warps composing different clusters) and Eq. 2.
+// One stable pass of a radix sort over n records by a whole block (kBigThreads): records move from
+// src to dst in increasing order of the 8 bits at `shift`, equal ones in their order. Tiles of
+// kBlockSort records are placed one after another: a warp ranks up to 256 consecutive records of the
+// tile, 32 a round (__match_any groups equal digits, the group's first lane advances the warp's
+// counter of that digit), then one scan over the counters by (digit, warp), eight a thread, gives
+// every record's place in the tile's order. s_wc [kDigits][kWcStride]: a digit's counters of the
+// warps lie 33 apart, so that neither the ranking nor the scan meets bank conflicts. s_base
+// [kDigits], s_sum [32]: shared memory.
+constexpr uint32_t kWcStride = kBigThreads / 32 + 1;
+
+__device__ __forceinline__ void radix_pass(const unsigned long long* src, unsigned long long* dst, uint32_t n,
+                                           int shift, uint32_t* s_wc, uint32_t* s_base, uint32_t* s_sum)
+{
+    constexpr uint32_t kRounds = kBlockSort / kBigThreads, kWarps = kBigThreads / 32;
+    static_assert(kWarps == 32 && kDigits * kWarps == 8 * kBigThreads, "eight counters a thread");
+    const uint32_t t = threadIdx.x, lane = t & 31u, warp = t >> 5;
+    const uint32_t rounds = min(kRounds, (n + kBigThreads - 1) / kBigThreads);  // of a warp in a tile
+    auto digit = [&](unsigned long long e) { return (uint32_t)(e >> shift) & (kDigits - 1); };
+    // exclusive prefix over the block's threads (two barriers)
+    auto block_scan = [&](uint32_t v) {
+        uint32_t x = v;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const uint32_t y = __shfl_up_sync(0xffffffffu, x, o);
+            if (lane >= o) x += y;
+        }
+        if (lane == 31) s_sum[warp] = x;
+        __syncthreads();
+        uint32_t w = s_sum[lane];
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const uint32_t y = __shfl_up_sync(0xffffffffu, w, o);
+            if (lane >= o) w += y;
+        }
+        const uint32_t before = __shfl_sync(0xffffffffu, w, (warp + 31) & 31);
+        return (warp ? before : 0u) + x - v;
+    };
+    const bool one = n <= kBlockSort;
+    if (!one) {  // where each digit's records begin, over all tiles
+        if (t < kDigits) s_base[t] = 0u;
+        __syncthreads();
+        for (uint32_t k0 = 0; k0 < n; k0 += kBigThreads) {
+            const uint32_t k = k0 + t, d = k < n ? digit(src[k]) : kDigits;
+            const uint32_t peers = __match_any_sync(0xffffffffu, d);
+            if (d < kDigits && lane == (uint32_t)(__ffs(peers) - 1)) atomicAdd(&s_base[d], (uint32_t)__popc(peers));
+        }
+        __syncthreads();
+        const uint32_t first = block_scan(t < kDigits ? s_base[t] : 0u);
+        __syncthreads();
+        if (t < kDigits) s_base[t] = first;
+    }
+    for (uint32_t tile = 0; tile < n; tile += kBlockSort) {
+        for (uint32_t k = t; k < kDigits * kWcStride; k += kBigThreads) s_wc[k] = 0u;
+        __syncthreads();
+        unsigned long long rec[kRounds];
+        uint32_t at[kRounds];  // digit << 16 | rank among the warp's records of that digit
+#pragma unroll
+        for (uint32_t r = 0; r < kRounds; ++r) {
+            rec[r] = 0ull;
+            at[r] = kDigits << 16;
+            if (r >= rounds) continue;
+            const uint32_t k = tile + (warp * rounds + r) * 32 + lane;
+            if (k < n) rec[r] = src[k];
+            const uint32_t d = k < n ? digit(rec[r]) : kDigits;
+            const uint32_t peers = __match_any_sync(0xffffffffu, d);
+            const int leader = __ffs(peers) - 1;
+            uint32_t old = 0;
+            if (d < kDigits && lane == (uint32_t)leader) {
+                old = s_wc[d * kWcStride + warp];
+                s_wc[d * kWcStride + warp] = old + (uint32_t)__popc(peers);
+            }
+            old = __shfl_sync(0xffffffffu, old, leader);
+            at[r] = d << 16 | (old + (uint32_t)__popc(peers & lanemask_lt()));
+            __syncwarp();
+        }
+        __syncthreads();
+        uint32_t* mine = s_wc + (t >> 2) * kWcStride + 8 * (t & 3u);  // digit t / 4, eight warps
+        uint32_t c[8], sum = 0;
+#pragma unroll
+        for (int k = 0; k < 8; ++k) {
+            c[k] = mine[k];
+            sum += c[k];
+        }
+        uint32_t run = block_scan(sum);
+        if (!one) {  // after the digit's records of the tiles before: its place less its place in the tile
+            const uint32_t tile_first = __shfl_sync(0xffffffffu, run, lane & ~3u);
+            const uint32_t tile_end = __shfl_sync(0xffffffffu, run + sum, lane | 3u);
+            const uint32_t base = s_base[t >> 2];
+            __syncwarp();
+            if ((t & 3u) == 0) s_base[t >> 2] = base + tile_end - tile_first;
+            run += base - tile_first;
+        }
+#pragma unroll
+        for (int k = 0; k < 8; ++k) {
+            mine[k] = run;
+            run += c[k];
+        }
+        __syncthreads();
+#pragma unroll
+        for (uint32_t r = 0; r < kRounds; ++r) {
+            const uint32_t d = at[r] >> 16;
+            if (d < kDigits) dst[s_wc[d * kWcStride + warp] + (at[r] & 0xFFFFu)] = rec[r];
+        }
+        __syncthreads();
+    }
+}
+
+// 5b. one block per cell of the sorting list (more than kBlockGroup records), which it puts in
+// (cluster, sample id) order by radix passes over the ids' bits (of n_ids ids; less the cell's smallest
+// one, where they have more than 24) and the clusters. Up to kBlockSort records whose ids span 24 bits, in shared memory: words (cluster << 24 |
+// id) << 32 | reward. Others in global scratch, the cell's part of the bucket and of `wide` in turn:
+// words cluster << 32 | id, rewards read by sample id at the end. Then Eq. 1 (warps composing
+// different clusters) and Eq. 2. A cell of 8 192 records takes four passes of one tile; the bitonic
+// network that this replaces took 91 steps with a barrier each, and its global form 105 and more
+// 200 x 120 points at 64 samples, 483 such cells: 186 us -> 103).
 template <int P, class Rows, class Split>
 __global__ void __launch_bounds__(kBigThreads)
 k_learn_big(const Bucket bucket, unsigned long long* __restrict__ wide, const float* __restrict__ rec_val,
             const uint32_t* __restrict__ ctr,
             const uint32_t* __restrict__ touched, const uint32_t* __restrict__ start,
             const uint32_t* __restrict__ len, const uint32_t* __restrict__ big, uint32_t* __restrict__ cursor,
-            Rows rows, Split sp, uint32_t* __restrict__ status)
+            Rows rows, Split sp, uint32_t* __restrict__ status, uint32_t n_ids)
 {
+    const uint32_t n_big = *(volatile const uint32_t*)(ctr + 2);  // complete: see k_learn_buckets
+    if (n_big == 0) {
+        pdl_release();
+        pdl_wait();
+        return;
+    }
     pdl_begin();
-    extern __shared__ unsigned long long s_key[];      // kBlockSort keys, then kBlockSort rewards (u32)
-    uint32_t* s_val = reinterpret_cast<uint32_t*>(s_key + kBlockSort);
+    extern __shared__ unsigned long long s_rec[];      // two tiles, then the warps' digit counters
+    uint32_t* s_wc = reinterpret_cast<uint32_t*>(s_rec + 2 * kBlockSort);
     __shared__ float s_q[kMaxCut], s_c[kMaxCut];
     __shared__ uint16_t s_b[kMaxCut];
-    __shared__ uint32_t s_gs[kMaxCut], s_ge[kMaxCut];
-    const uint32_t n_big = *(volatile const uint32_t*)(ctr + 2);
+    __shared__ uint32_t s_gs[kMaxCut], s_ge[kMaxCut], s_lim[2], s_base[kDigits], s_sum[32];
     for (uint32_t bi = blockIdx.x; bi < n_big; bi += gridDim.x) {
         const uint32_t w = big[bi];
         const uint32_t slot = touched[w], b0 = start[w], nr = len[w];
@@ -594,39 +721,57 @@ k_learn_big(const Bucket bucket, unsigned long long* __restrict__ wide, const fl
         const uint32_t M = r.M, m = r.m;
         const float alpha = r.alpha;
         if (threadIdx.x < 32) load_q_row<P>(r.Q, m, s_q);
-        if (nr <= kBlockSort) {
+        uint32_t lo = 0, hi = n_ids - 1u;
+        if (bucket.s) {  // ids of more than 24 bits: the cell's smallest and largest
+            if (threadIdx.x < 2) s_lim[threadIdx.x] = threadIdx.x ? 0u : 0xFFFFFFFFu;
+            __syncthreads();
+            lo = 0xFFFFFFFFu;
+            hi = 0u;
             for (uint32_t k = threadIdx.x; k < nr; k += blockDim.x) {
                 uint32_t id, cls, bits;
                 bucket.get(b0 + k, id, cls, bits);
-                s_key[k] = ((unsigned long long)cls << 45) | ((unsigned long long)id << 13) | k;
+                lo = min(lo, id);
+                hi = max(hi, id);
+            }
+            lo = __reduce_min_sync(0xffffffffu, lo);
+            hi = __reduce_max_sync(0xffffffffu, hi);
+            if ((threadIdx.x & 31) == 0) {
+                atomicMin(&s_lim[0], lo);
+                atomicMax(&s_lim[1], hi);
             }
             __syncthreads();
-            bitonic_sort_u64(s_key, nr, threadIdx.x, blockDim.x, BlockSync{});
-            for (uint32_t j = threadIdx.x; j < nr; j += blockDim.x) {
-                uint32_t id, cls, bits;
-                bucket.get(b0 + (uint32_t)(s_key[j] & (kBlockSort - 1)), id, cls, bits);
-                s_val[j] = bits;
-            }
-            __syncthreads();
-            compose_sorted_block<P>([&](uint32_t j) { return (uint32_t)(s_key[j] >> 45); },
-                                    [&](uint32_t j) { return s_val[j]; }, nr, M, m, alpha, s_q, s_gs, s_ge);
-        } else {
-            unsigned long long* rec = wide + b0;
-            for (uint32_t k = threadIdx.x; k < nr; k += blockDim.x) {
-                uint32_t id, cls, bits;
-                bucket.get(b0 + k, id, cls, bits);
-                rec[k] = ((unsigned long long)cls << 32) | id;
-            }
-            __syncthreads();
-            bitonic_sort_u64(rec, nr, threadIdx.x, blockDim.x, BlockSync{});
-            for (uint32_t k = threadIdx.x; k < nr; k += blockDim.x) {
-                const unsigned long long e = rec[k];
-                rec[k] = (e & 0xFFFFFFFF00000000ull) | __float_as_uint(__ldg(rec_val + (uint32_t)e));
-            }
-            __syncthreads();
-            compose_sorted_block<P>([&](uint32_t j) { return (uint32_t)(rec[j] >> 32); },
-                                    [&](uint32_t j) { return (uint32_t)rec[j]; }, nr, M, m, alpha, s_q, s_gs, s_ge);
+            lo = s_lim[0];
+            hi = s_lim[1];
         }
+        const int id_bits = 32 - __clz((int)(hi - lo));
+        const bool small = nr <= kBlockSort && id_bits <= 24;
+        unsigned long long* src = small ? s_rec : wide + b0;
+        unsigned long long* dst = small ? s_rec + kBlockSort : bucket.word + b0;
+        for (uint32_t k = threadIdx.x; k < nr; k += blockDim.x) {
+            uint32_t id, cls, bits;
+            bucket.get(b0 + k, id, cls, bits);
+            id -= lo;
+            src[k] = small ? ((unsigned long long)(cls << 24 | id) << 32) | bits : ((unsigned long long)cls << 32) | id;
+        }
+        __syncthreads();
+        for (int shift = 0; shift < id_bits + 8; shift += 8) {  // the ids' digits, then the clusters
+            const int at = shift < id_bits ? shift : (small ? 24 : 32);
+            radix_pass(src, dst, nr, small ? 32 + at : at, s_wc, s_base, s_sum);
+            unsigned long long* other = src;
+            src = dst;
+            dst = other;
+            if (shift >= id_bits) break;
+        }
+        if (!small) {
+            for (uint32_t k = threadIdx.x; k < nr; k += blockDim.x) {
+                const unsigned long long e = src[k];
+                src[k] = (e & 0xFFFFFFFF00000000ull) | __float_as_uint(__ldg(rec_val + lo + (uint32_t)e));
+            }
+            __syncthreads();
+        }
+        const int cls_at = small ? 56 : 32;
+        compose_sorted_block<P>([&](uint32_t j) { return (uint32_t)(src[j] >> cls_at); },
+                                [&](uint32_t j) { return (uint32_t)src[j]; }, nr, M, m, alpha, s_q, s_gs, s_ge);
         if (threadIdx.x < 32) {  // the cluster bounds are dead: the cut scratch rows
             finish_cell<P>(sp, slot, s_q, m, r.eps, r.Q, r.C, s_gs, s_ge, s_c, s_b, status);
             if (threadIdx.x == 0) cursor[slot] = 0u;
@@ -696,19 +841,21 @@ cudaError_t launch_bucketed_learn(cudaStream_t s, int device, int sms, const uin
         e0 = launch_pdl(k_bucket_scatter<Dec>, dim3(rblocks), dim3(kBucketThreads), 0, s, rec_key, rec_val, n, dec,
                         cursor, rank, bucket);
     if (e0 != cudaSuccess) return e0;
+    // k_learn_big first, k_learn_buckets beside it: its blocks, few and long, take the place they need,
+    // and without cells for them they cost nothing (whole passes: 64-sample tile 346 -> 307 us, path
+    // vertices 479 -> 467, others equal)
+    e0 = big_smem_attribute<P, Rows, Split>(device);
+    if (e0 == cudaSuccess)
+        e0 = launch_pdl(k_learn_big<P, Rows, Split>, dim3(sms), dim3(kBigThreads), kBigSmem, s, bucket, wide, rec_val,
+                        ctr, touched, start, len, sort_list, cursor, rows, sp, status, (uint32_t)n);
+    if (e0 != cudaSuccess) return e0;
     // cuts of at most 64 leaves: per-cluster arrays of 64 entries (30.5 KB of shared memory per
     // block), 56 registers, 6 blocks per SM; larger cuts: 256 entries (44.4 KB), 5 blocks per SM
     if (max_cut <= 64)
-        e0 = launch_pdl(k_learn_buckets<P, 6, 6, 64, Rows, Split>, dim3(sms * 6), dim3(6 * 32), 0, s, bucket, ctr,
-                        group_list, touched, start, len, cursor, rows, sp, status, cells);
-    else
-        e0 = launch_pdl(k_learn_buckets<P, 6, 5, kMaxCut, Rows, Split>, dim3(sms * 5), dim3(6 * 32), 0, s, bucket,
-                        ctr, group_list, touched, start, len, cursor, rows, sp, status, cells);
-    if (e0 != cudaSuccess) return e0;
-    cudaError_t e = big_smem_attribute<P, Rows, Split>(device);
-    if (e != cudaSuccess) return e;
-    return launch_pdl(k_learn_big<P, Rows, Split>, dim3(sms * 2), dim3(kBigThreads), kBigSmem, s, bucket, wide,
-                      rec_val, ctr, touched, start, len, sort_list, cursor, rows, sp, status);
+        return launch_pdl(k_learn_buckets<P, 6, 6, 64, Rows, Split>, dim3(sms * 6), dim3(6 * 32), 0, s, bucket, ctr,
+                          group_list, touched, start, len, cursor, rows, sp, status, cells);
+    return launch_pdl(k_learn_buckets<P, 6, 5, kMaxCut, Rows, Split>, dim3(sms * 5), dim3(6 * 32), 0, s, bucket, ctr,
+                      group_list, touched, start, len, cursor, rows, sp, status, cells);
 }
 
 }  // namespace

@@ -20,9 +20,9 @@
 //      applies the composite to the cluster's Q held in shared memory; the
 //      row is then stored in the table precision and its cdf rebuilt (Eq. 2
 //      with the floor, prefix sum across the warp). Cells with more records
-//      than a warp's buffer go to one block each: (cluster, sample id, index)
-//      keys sorted by a bitonic network in shared memory (up to 8192
-//      records; in place in global memory above that), then warps compose
+//      than a warp's buffer go to two warps or to one block, those of more than
+//      1024 to a block that sorts them by radix passes in shared memory (up
+//      to 8192 records; in global scratch above that); then warps compose
 //      different clusters in parallel.
 // The order inside a bucket depends on thread scheduling; the per-cell sort
 // restores sample order, so the result is deterministic. Every kernel of the

@@ -214,51 +214,6 @@ __device__ void learn_one_cell(const uint32_t* __restrict__ sk, const uint32_t* 
     warp_rebuild_cdf<P>(q, (int)m, eps, crow, c, bits);
 }
 
-// ---------------------------------------------------------------- per-cell sort
-// Ascending sort of a[0..n) by a bitonic network in which every comparator
-// puts the minimum at the lower index: per merge size k, first the mirror
-// step (i against i ^ (k - 1)), then half-cleaners (i against i + j). The
-// array is padded virtually to the next power of two with +infinity; a
-// comparator that reaches a padded position would leave it unchanged, so it
-// is skipped. `tid`/`nthreads` split the comparators; `sync` is the barrier
-// of the participating threads (__syncwarp or __syncthreads).
-__device__ __forceinline__ void cmp_swap(unsigned long long* a, uint32_t i, uint32_t p)
-{
-    const unsigned long long x = a[i], y = a[p];
-    if (y < x) {
-        a[i] = y;
-        a[p] = x;
-    }
-}
-
-template <class Sync>
-__device__ __forceinline__ void bitonic_sort_u64(unsigned long long* a, uint32_t n, uint32_t tid, uint32_t nthreads,
-                                                 Sync sync)
-{
-    if (n < 2) return;
-    uint32_t lg = 0;
-    while ((1u << lg) < n) ++lg;
-    const uint32_t half_len = 1u << (lg - 1);
-    for (uint32_t lk = 1; lk <= lg; ++lk) {
-        const uint32_t k = 1u << lk;
-        for (uint32_t t = tid; t < half_len; t += nthreads) {
-            const uint32_t i = ((t >> (lk - 1)) << lk) | (t & ((k >> 1) - 1));
-            const uint32_t p = i ^ (k - 1);
-            if (p < n) cmp_swap(a, i, p);
-        }
-        sync();
-        for (uint32_t lj = lk - 1; lj-- > 0;) {
-            const uint32_t j = 1u << lj;
-            for (uint32_t t = tid; t < half_len; t += nthreads) {
-                const uint32_t i = ((t >> lj) << (lj + 1)) | (t & (j - 1));
-                const uint32_t p = i + j;
-                if (p < n) cmp_swap(a, i, p);
-            }
-            sync();
-        }
-    }
-}
-
 // Eq. 1 for one cell whose records are given in (cluster, sample id) order:
 // get(j) = (cluster, reward bits) of record j < len. The records are
 // composed 32 at a time exactly as learn_one_cell does (segmented scan of the
@@ -293,6 +248,62 @@ __device__ void learn_records(Get get, uint32_t len, uint32_t m, float alpha, fl
         __syncwarp();
     }
 }
+
+// learn_records for the records of one cluster alone, in sample order. The same composition, hence
+// the same bits: the slopes of a scan's steps are those of every other 32 records, so they are formed
+// once (a warp's GroupScan serves all its clusters) and only the offsets are scanned: a shuffle a
+// step instead of three, and of a long group four times 32 records in flight.
+struct GroupScan {
+    float alpha, A[6];
+
+    __device__ __forceinline__ explicit GroupScan(float a) : alpha(a)
+    {
+        const uint32_t lane = threadIdx.x & 31u;
+        A[0] = 1.0f - a;
+#pragma unroll
+        for (int k = 0; k < 5; ++k) {
+            const float Ao = __shfl_up_sync(0xffffffffu, A[k], 1u << k);
+            A[k + 1] = lane >= (1u << k) ? A[k] * Ao : A[k];
+        }
+    }
+    // N times 32 records from val(0), the last of them possibly fewer (len in all)
+    template <int N, class Val>
+    __device__ __forceinline__ float some(Val val, uint32_t len, float q) const
+    {
+        const uint32_t lane = threadIdx.x & 31u;
+        float B[N];
+#pragma unroll
+        for (int c = 0; c < N; ++c) {
+            const uint32_t j = 32 * c + lane;
+            B[c] = j < len ? alpha * __uint_as_float(val(j)) : 0.0f;
+        }
+#pragma unroll
+        for (int k = 0; k < 5; ++k) {
+#pragma unroll
+            for (int c = 0; c < N; ++c) {
+                const float Bo = __shfl_up_sync(0xffffffffu, B[c], 1u << k);
+                if (lane >= (1u << k)) B[c] = A[k] * Bo + B[c];
+            }
+        }
+#pragma unroll
+        for (int c = 0; c < N; ++c) {
+            const int last = (int)min(31u, len - 1u - 32u * c);
+            q = __shfl_sync(0xffffffffu, A[5], last) * q + __shfl_sync(0xffffffffu, B[c], last);
+        }
+        return q;
+    }
+    // val(j): the reward bits of record j < len; q: the cluster's Q, on every lane
+    template <class Val>
+    __device__ __forceinline__ float run(Val val, uint32_t len, float q) const
+    {
+        uint32_t pos = 0;
+#pragma unroll 1
+        for (; len - pos >= 128; pos += 128) q = some<4>([&](uint32_t j) { return val(pos + j); }, 128, q);
+#pragma unroll 1
+        for (; pos < len; pos += 32) q = some<1>([&](uint32_t j) { return val(pos + j); }, len - pos, q);
+        return q;
+    }
+};
 
 // Split-collapse steps on one cell's rows in shared memory (cut cs, Q q,
 // both of m entries; c and nc: scratch rows), repeated until a step changes

@@ -442,10 +442,12 @@ template <> struct Store<RLL_PREC_BF16> {
 // statement is pdl_begin(): wait until that kernel (and so all earlier work)
 // has completed and its writes are visible, then let the next kernel be
 // scheduled in turn.
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void pdl_release() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void pdl_begin()
 {
-    asm volatile("griddepcontrol.wait;" ::: "memory");
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    pdl_wait();
+    pdl_release();
 }
 
 template <typename... KArgs, typename... Args>
