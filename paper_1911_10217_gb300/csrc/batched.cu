@@ -496,6 +496,7 @@ int rll_batch_set_items(rll_ctx* ctx, rll_batch* b, const rll_batch_item* items,
         a.pairs = t->pairs;
         a.tail_tex = t->tail_tex;
         a.quads = t->quads;
+        a.quad_tex = t->quad_tex;
         a.nodes = t->nodes;
         a.lights = t->lights;
         a.light_cdf = t->light_cdf;

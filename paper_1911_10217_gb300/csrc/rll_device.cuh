@@ -44,10 +44,9 @@ struct __align__(16) NodeRec {
 };
 static_assert(sizeof(NodeRec) == 64, "NodeRec must be 64 bytes");
 
-// Descent record of one child, 48 bytes: the constants of the importance
-// bound precomputed (binary32, same operations as on the fly). The two-level
-// descent reads them four per internal node (quads).
-struct __align__(16) DescRec {
+// Descent constants of a node: the importance bound's, precomputed (binary32,
+// same operations as on the fly).
+struct DescRec {
     float c[3];      // AABB centre
     float r2;        // squared half diagonal
     float r;         // half diagonal
@@ -57,7 +56,6 @@ struct __align__(16) DescRec {
     float sin_t;     // cone sin(theta)
     uint32_t id;     // node id
 };
-static_assert(sizeof(DescRec) == 48, "DescRec must be 48 bytes");
 
 // The DescRec fields of both children of one internal node, interleaved
 // (x: left child, y: right child) so that a load yields packed operands of
@@ -84,6 +82,17 @@ struct __align__(16) PairTail {
     uint32_t id[2];
 };
 static_assert(sizeof(PairTail) == 16, "PairTail must be 16 bytes");
+
+// The two-level descent's candidates below one internal node, two and two as
+// above, and their powers and ids (two texels).
+struct __align__(32) QuadRec {
+    PairRec pair[2];
+};
+struct __align__(16) QuadTail {
+    float phi[4];
+    uint32_t id[4];
+};
+static_assert(sizeof(QuadRec) == 128 && sizeof(QuadTail) == 32, "two-level record sizes");
 
 // Sorted light, 64 bytes (two 256-bit loads).
 struct __align__(32) LightRec {
@@ -269,29 +278,13 @@ __device__ __forceinline__ DescRec make_desc(const NodeRec& n)
 // and emitter cosine bounds over the node's bounding sphere, over distance^2,
 // kept as num / den = (phi A B) / d^6 with A = d^2 Brecv, B = d^2 Bemit.
 // Cosines and sines are carried multiplied by |d| (2-3 square roots, no
-// division).
-struct Bound {
-    float num, den;
-};
-
-__device__ __forceinline__ Bound importance(const DescRec& r, float x0, float x1, float x2, float n0, float n1,
-                                            float n2)
-{
-    const float dx = fsub(r.c[0], x0), dy = fsub(r.c[1], x1), dz = fsub(r.c[2], x2);
-    const float d2 = __fmaf_rn(dz, dz, __fmaf_rn(dy, dy, fmul(dx, dx)));
-    if (d2 <= r.r2) return Bound{r.phi, fmaxf(r.r2, 1e-30f)};
-    const float cb = fsqrt(fsub(d2, r.r2));
-    const float nd = __fmaf_rn(n2, dz, __fmaf_rn(n1, dy, fmul(n0, dx)));
-    float A = d2;
-    if (nd < cb) A = fmaxf(0.0f, __fmaf_rn(nd, cb, fmul(fsqrt(fmaxf(0.0f, __fmaf_rn(-nd, nd, d2))), r.r)));
-    const float ad = -__fmaf_rn(r.axis[2], dz, __fmaf_rn(r.axis[1], dy, fmul(r.axis[0], dx)));
-    const float sphi = __fmaf_rn(r.sin_t, cb, fmul(r.cos_t, r.r));
-    const float cphi = __fmaf_rn(r.cos_t, cb, -fmul(r.sin_t, r.r));
-    float B = d2;
-    if (!(sphi <= 0.0f || cphi <= ad))
-        B = fmaxf(0.0f, __fmaf_rn(ad, cphi, fmul(fsqrt(fmaxf(0.0f, __fmaf_rn(-ad, ad, d2))), sphi)));
-    return Bound{fmul(fmul(r.phi, A), B), fmul(fmul(d2, d2), d2)};
-}
+// division). For a node at d = c - x (d2 = |d|^2):
+//   d2 <= r2: num = phi, den = max(r2, 1e-30); else
+//   cb = sqrt(d2 - r2); nd = n d; A = nd < cb ? max(0, nd cb + sqrt(max(0, d2 - nd^2)) r) : d2;
+//   ad = -axis d; sphi = sin cb + cos r; cphi = cos cb - sin r;
+//   B = sphi <= 0 or cphi <= ad ? d2 : max(0, ad cphi + sqrt(max(0, d2 - ad^2)) sphi);
+//   num = (phi A) B; den = (d2 d2) d2,
+// sums of products from the left, each but the first product fused (x, y, z in turn).
 
 // Correctly rounded square root of two values at once, sign-flipped: for n = -x (x in {0} or
 // [2^-100, 2^60), else see below) returns -sqrt(x), bit for bit __fsqrt_rn's value. One
@@ -318,9 +311,8 @@ __device__ __forceinline__ float2 neg_sqrt2(float2 n)
     return __ffma2_rn(e, h, s);
 }
 
-// importance() of both children of a node at once, in packed binary32
-// (f32x2) arithmetic: per component the same correctly rounded operations in
-// the same order as importance(), hence bit-identical bounds. Signs are folded
+// The importance of two nodes at once, in packed binary32 (f32x2) arithmetic:
+// per component the correctly rounded operations above in their order. Signs are folded
 // into the operands (rounding to nearest is symmetric), since a packed
 // instruction takes no sign modifier: nt = r2 - d2, ncb = -cb, g = nd^2 - d2,
 // nad = -ad, nsp = -sphi, ncp = -cphi. The early return inside the bounding

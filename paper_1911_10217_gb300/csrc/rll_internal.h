@@ -11,7 +11,8 @@
 
 namespace rll {
 struct NodeRec;
-struct DescRec;
+struct QuadRec;
+struct QuadTail;
 struct PairRec;
 struct PairTail;
 struct LightRec;
@@ -51,8 +52,10 @@ struct rll_tree {
     rll::PairRec* pairs = nullptr;   // [n-1] geometry of both children of internal i, interleaved
     rll::PairTail* tails = nullptr;  // [n-1] their powers and ids
     cudaTextureObject_t tail_tex = 0; // tails as float4 texels (n > 1)
-    rll::DescRec* quads = nullptr;   // [4(n-1)] records of the 2..4 grandchildren of internal i at 4i.. (two-level
-                                     // descent; a single-light child stands for itself; unused entries id ~0)
+    rll::QuadRec* quads = nullptr;       // [n-1] geometry of the 2..4 grandchildren of internal i (two-level descent;
+                                         // a single-light child stands for itself)
+    rll::QuadTail* quad_tails = nullptr; // [n-1] their powers and ids (unused candidates: id ~0)
+    cudaTextureObject_t quad_tex = 0;    // quad_tails as float4 texels (n > 1)
     rll::LightRec* lights = nullptr; // [n] sorted lights
     uint32_t* perm = nullptr;        // [n] sorted -> input index
     int32_t* left = nullptr;         // [n-1]

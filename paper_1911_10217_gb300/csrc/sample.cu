@@ -208,6 +208,7 @@ int sample_and_shade_range(rll_ctx* ctx, rll_grid* g, const rll_tree* t, const f
     a.pairs = t->pairs;
     a.tail_tex = t->tail_tex;
     a.quads = t->quads;
+    a.quad_tex = t->quad_tex;
     a.nodes = t->nodes;
     a.lights = t->lights;
     a.light_cdf = t->light_cdf;

@@ -38,7 +38,8 @@ struct SampleArgs {
     uint32_t reward_mode;
     const PairRec* pairs;
     cudaTextureObject_t tail_tex;  // the pairs' powers and ids
-    const DescRec* quads;     // two-level descent records (4 per internal node)
+    const QuadRec* quads;     // two-level descent records
+    cudaTextureObject_t quad_tex;  // the quads' powers and ids
     const NodeRec* nodes;
     const LightRec* lights;
     const float* light_cdf;
@@ -90,14 +91,14 @@ __device__ __forceinline__ int64_t lookup_insert(unsigned long long* keys, uint3
     return -1;
 }
 
-__device__ __forceinline__ DescRec load_desc(const DescRec* p)
+// the geometry of two nodes
+__device__ __forceinline__ NodePair load_pair(const PairRec* p)
 {
-    DescRec r;
-    const float4* s = reinterpret_cast<const float4*>(p);
-    float4* d = reinterpret_cast<float4*>(&r);
-#pragma unroll
-    for (int k = 0; k < 3; ++k) d[k] = __ldg(s + k);
-    return r;
+    const Words8 u = ldg_words8(p), v = ldg_words8(reinterpret_cast<const char*>(p) + 32);
+    auto pair = [](const Words8& w, int k) {
+        return make_float2(__uint_as_float(w.w[2 * k]), __uint_as_float(w.w[2 * k + 1]));
+    };
+    return NodePair{pair(u, 0), pair(u, 1), pair(u, 2), pair(u, 3), pair(v, 0), pair(v, 1), pair(v, 2), v.w[6], v.w[7]};
 }
 
 __device__ __forceinline__ LightRec load_light(const LightRec* p)
@@ -260,12 +261,7 @@ __device__ __forceinline__ void descent_step(const SampleArgs& a, uint32_t& node
                                              float2 nx0, float2 nx1, float2 nx2, float2 n0, float2 n1, float2 n2)
 {
     const float4 t = tex1Dfetch<float4>(a.tail_tex, (int)node);  // powers, then ids
-    const Words8 u = ldg_words8(a.pairs + node), v = ldg_words8(reinterpret_cast<const char*>(a.pairs + node) + 32);
-    auto pair = [](const Words8& w, int k) {
-        return make_float2(__uint_as_float(w.w[2 * k]), __uint_as_float(w.w[2 * k + 1]));
-    };
-    const NodePair q{pair(u, 0), pair(u, 1), pair(u, 2), pair(u, 3), pair(v, 0), pair(v, 1), pair(v, 2), v.w[6], v.w[7]};
-    const Bound2 b = importance2(q, make_float2(t.x, t.y), nx0, nx1, nx2, n0, n1, n2);
+    const Bound2 b = importance2(load_pair(a.pairs + node), make_float2(t.x, t.y), nx0, nx1, nx2, n0, n1, n2);
     float wl = fmul(b.num.x, b.den.y), wr = fmul(b.num.y, b.den.x);
     float ssum = fadd(wl, wr);
     if (!(ssum > 0.0f)) {
@@ -286,50 +282,39 @@ __device__ __forceinline__ void descent_step(const SampleArgs& a, uint32_t& node
     node = __float_as_uint(left ? t.z : t.w);
 }
 
-__device__ __forceinline__ void prefetch_l1(const void* p)
-{
-    asm volatile("prefetch.global.L1 [%0];" ::"l"(p));
-}
-
 // One step of the two-level descent below internal node `node` (ud: the
-// step's draw): candidates quads[4 node ..] (2 to 4 valid, in light order),
-// weights num / max(den, 1e-30), binary32 prefix sums in order; the first
+// step's draw): its candidates (2 to 4 valid, in light order, the valid ones
+// first), weights num / max(den, 1e-30), binary32 prefix sums in order; the first
 // prefix above u * S is chosen (exact, one fma), probability (P_i -
 // P_{i-1}) / S; powers, then uniform over the valid candidates, when all
-// weights vanish. Candidates 2 and 3 are prefetched into L1 while 0 and 1
-// are evaluated, so no registers hold them meanwhile.
-__device__ __forceinline__ void descent2_step(const SampleArgs& a, uint32_t& node, float& p_in, float ud, float x0,
-                                              float x1, float x2, float n0, float n1, float n2)
+// weights vanish. Two candidates a bound, from four 32-byte loads and two
+// texels (one candidate a bound from twelve 16-byte loads of 48-byte records:
+// 1 601 x 901 points, binary16 tables: 369 us a pass, now 312).
+__device__ __forceinline__ void descent2_step(const SampleArgs& a, uint32_t& node, float& p_in, float ud, float2 nx0,
+                                              float2 nx1, float2 nx2, float2 n0, float2 n1, float2 n2)
 {
-    const DescRec* q = a.quads + 4 * (int64_t)node;
-    prefetch_l1(q + 2);
-    prefetch_l1(reinterpret_cast<const char*>(q + 2) + 64);
-    float w[4];
-    bool valid3 = false, valid4 = false;
-#pragma unroll
-    for (int h = 0; h < 2; ++h) {
-        const DescRec A = load_desc(q + 2 * h), B = load_desc(q + 2 * h + 1);
-        const Bound ba = importance(A, x0, x1, x2, n0, n1, n2);
-        const Bound bb = importance(B, x0, x1, x2, n0, n1, n2);
-        w[2 * h] = fdiv(ba.num, fmaxf(ba.den, 1e-30f));
-        w[2 * h + 1] = fdiv(bb.num, fmaxf(bb.den, 1e-30f));
-        if (h == 1) {
-            valid3 = A.id != 0xFFFFFFFFu;
-            valid4 = B.id != 0xFFFFFFFFu;
-        }
-    }
-    const int k = 2 + valid3 + valid4;  // valid candidates come first
+    const float4 phi = tex1Dfetch<float4>(a.quad_tex, (int)(2 * node));
+    const float4 idf = tex1Dfetch<float4>(a.quad_tex, (int)(2 * node + 1));
+    const uint32_t id[4] = {__float_as_uint(idf.x), __float_as_uint(idf.y), __float_as_uint(idf.z),
+                            __float_as_uint(idf.w)};
+    const QuadRec* q = a.quads + node;
+    const Bound2 b0 = importance2(load_pair(&q->pair[0]), make_float2(phi.x, phi.y), nx0, nx1, nx2, n0, n1, n2);
+    const Bound2 b1 = importance2(load_pair(&q->pair[1]), make_float2(phi.z, phi.w), nx0, nx1, nx2, n0, n1, n2);
+    const int k = 2 + (id[2] != 0xFFFFFFFFu) + (id[3] != 0xFFFFFFFFu);
+    const float w[4] = {fdiv(b0.num.x, fmaxf(b0.den.x, 1e-30f)), fdiv(b0.num.y, fmaxf(b0.den.y, 1e-30f)),
+                        fdiv(b1.num.x, fmaxf(b1.den.x, 1e-30f)), fdiv(b1.num.y, fmaxf(b1.den.y, 1e-30f))};
     float pre[4], S = 0.0f;
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
         S = fadd(S, i < k ? w[i] : 0.0f);
         pre[i] = S;
     }
-    if (!(S > 0.0f)) {  // rare: the candidates' powers (read again, L1)
+    if (!(S > 0.0f)) {  // rare: the candidates' powers
+        const float power[4] = {phi.x, phi.y, phi.z, phi.w};
         S = 0.0f;
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
-            S = fadd(S, i < k ? __ldg(&q[i].phi) : 0.0f);
+            S = fadd(S, i < k ? power[i] : 0.0f);
             pre[i] = S;
         }
     }
@@ -343,17 +328,18 @@ __device__ __forceinline__ void descent2_step(const SampleArgs& a, uint32_t& nod
         const uint32_t u24v = (uint32_t)(ud * 16777216.0f);
         pick = (int)(((unsigned long long)u24v * (unsigned long long)k) >> 24);
     }
-    // the chosen candidate's interval by selects (no indexed arrays), its id from L1
+    // the chosen candidate's interval and id by selects (no indexed arrays)
     float lo = 0.0f, hi = pre[0];
+    node = id[0];
 #pragma unroll
     for (int i = 1; i < 4; ++i) {
         if (pick == i) {
             lo = pre[i - 1];
             hi = pre[i];
+            node = id[i];
         }
     }
     p_in *= S > 0.0f ? (hi - lo) / S : 1.0f / (float)k;  // continuous: pdf only
-    node = __ldg(&q[pick].id);
 }
 
 // Light index of the node a descent ended on. A descent that ran into the
@@ -394,6 +380,8 @@ __device__ __forceinline__ void sample_one(const SampleArgs& a, const Point& pt,
     uint32_t node = su.node;
     float p_in = 1.0f;
     int64_t light;
+    const float2 vn0 = make_float2(n0, n0), vn1 = make_float2(n1, n1), vn2 = make_float2(n2, n2);
+    const float2 vx0 = make_float2(-x0, -x0), vx1 = make_float2(-x1, -x1), vx2 = make_float2(-x2, -x2);
     if (MODE == RLL_MODE_UNIFORM) {
         const NodeRec& r = a.nodes[node];
         const uint32_t w = r.end - r.begin;
@@ -401,12 +389,18 @@ __device__ __forceinline__ void sample_one(const SampleArgs& a, const Point& pt,
         light = (int64_t)r.begin + (int64_t)(((unsigned long long)u24v * w) >> 24);
         p_in = 1.0f / (float)w;
     } else if (MODE == RLL_MODE_DESCENT2) {
-        for (uint32_t level = 0; node < nl1u && level < (uint32_t)kMaxTreeDepth; ++level)
-            descent2_step(a, node, p_in, rs.draw(kDrawDescent + level), x0, x1, x2, n0, n1, n2);
+        // step l takes draw kDrawDescent + l, one copy of the step, the words rotated
+        uint4 w = su.w2;
+#pragma unroll 1
+        for (uint32_t l = 0; node < nl1u && l < (uint32_t)kMaxTreeDepth; ++l) {
+            const uint32_t k = (kDrawDescent + l) & 3u;
+            if (k == 0) w = rs.block_words((kDrawDescent + l) >> 2);
+            const float ud = u24(k == 0 ? w.x : w.y);
+            if (k != 0) w = make_uint4(0u, w.z, w.w, 0u);
+            descent2_step(a, node, p_in, ud, vx0, vx1, vx2, vn0, vn1, vn2);
+        }
         light = leaf_or_flag(a, node, nl1);
     } else {
-        const float2 vn0 = make_float2(n0, n0), vn1 = make_float2(n1, n1), vn2 = make_float2(n2, n2);
-        const float2 vx0 = make_float2(-x0, -x0), vx1 = make_float2(-x1, -x1), vx2 = make_float2(-x2, -x2);
         // Level l takes draw kDrawDescent + l: words 1..3 of Philox block 2, then four levels per block.
         // Five copies of the step in all: the first three levels share one, the rest are unrolled so
         // that every word index is a constant. The kernel's length counts: with seven copies, each

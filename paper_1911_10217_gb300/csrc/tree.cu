@@ -264,6 +264,24 @@ __global__ void k_finalize(int64_t nn, NodeRec* __restrict__ nodes, const int* _
     nodes[i].cos_t = fmaxf(-1.0f, ordered_to_float(cosmin[i]));
 }
 
+// the descent constants of two nodes, interleaved
+__device__ __forceinline__ PairRec pair_rec(const DescRec& L, const DescRec& R)
+{
+    PairRec q;
+    q.c0 = make_float2(L.c[0], R.c[0]);
+    q.c1 = make_float2(L.c[1], R.c[1]);
+    q.c2 = make_float2(L.c[2], R.c[2]);
+    q.r = make_float2(L.r, R.r);
+    q.a0 = make_float2(L.axis[0], R.axis[0]);
+    q.a1 = make_float2(L.axis[1], R.axis[1]);
+    q.a2 = make_float2(L.axis[2], R.axis[2]);
+    // exact: 1 - cos theta and sin theta are binary16 numbers
+    const __half2 hl = __halves2half2(__float2half_rn(fsub(1.0f, L.cos_t)), __float2half_rn(L.sin_t));
+    const __half2 hr = __halves2half2(__float2half_rn(fsub(1.0f, R.cos_t)), __float2half_rn(R.sin_t));
+    q.cs = make_uint2(*reinterpret_cast<const uint32_t*>(&hl), *reinterpret_cast<const uint32_t*>(&hr));
+    return q;
+}
+
 __global__ void k_pairs(int64_t n, const NodeRec* __restrict__ nodes, const int32_t* __restrict__ left,
                         const int32_t* __restrict__ right, PairRec* __restrict__ pairs, PairTail* __restrict__ tails,
                         float* __restrict__ leaf_phi)
@@ -271,20 +289,7 @@ __global__ void k_pairs(int64_t n, const NodeRec* __restrict__ nodes, const int3
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i < n - 1) {
         const DescRec L = make_desc(nodes[left[i]]), R = make_desc(nodes[right[i]]);
-        PairRec q;
-        q.c0 = make_float2(L.c[0], R.c[0]);
-        q.c1 = make_float2(L.c[1], R.c[1]);
-        q.c2 = make_float2(L.c[2], R.c[2]);
-        q.r = make_float2(L.r, R.r);
-        q.a0 = make_float2(L.axis[0], R.axis[0]);
-        q.a1 = make_float2(L.axis[1], R.axis[1]);
-        q.a2 = make_float2(L.axis[2], R.axis[2]);
-        {  // exact: 1 - cos theta and sin theta are binary16 numbers
-            const __half2 hl = __halves2half2(__float2half_rn(fsub(1.0f, L.cos_t)), __float2half_rn(L.sin_t));
-            const __half2 hr = __halves2half2(__float2half_rn(fsub(1.0f, R.cos_t)), __float2half_rn(R.sin_t));
-            q.cs = make_uint2(*reinterpret_cast<const uint32_t*>(&hl), *reinterpret_cast<const uint32_t*>(&hr));
-        }
-        pairs[i] = q;
+        pairs[i] = pair_rec(L, R);
         tails[i] = PairTail{{L.phi, R.phi}, {L.id, R.id}};
     }
     if (i < n) leaf_phi[i] = nodes[n - 1 + i].phi;
@@ -292,7 +297,7 @@ __global__ void k_pairs(int64_t n, const NodeRec* __restrict__ nodes, const int3
 
 // candidates of the two-level descent below internal node i, in light order
 __global__ void k_quads(int64_t n, const NodeRec* __restrict__ nodes, const int32_t* __restrict__ left,
-                        const int32_t* __restrict__ right, DescRec* __restrict__ quads)
+                        const int32_t* __restrict__ right, QuadRec* __restrict__ quads, QuadTail* __restrict__ tails)
 {
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n - 1) return;
@@ -308,12 +313,17 @@ __global__ void k_quads(int64_t n, const NodeRec* __restrict__ nodes, const int3
             cand[k++] = right[x];
         }
     }
+    DescRec d[4];
+    QuadTail t;
     for (int j = 0; j < 4; ++j) {
-        DescRec d{};
-        if (j < k) d = make_desc(nodes[cand[j]]);
-        else d.id = 0xFFFFFFFFu;
-        quads[4 * i + j] = d;
+        d[j] = DescRec{};
+        if (j < k) d[j] = make_desc(nodes[cand[j]]);
+        t.phi[j] = d[j].phi;
+        t.id[j] = j < k ? d[j].id : 0xFFFFFFFFu;
     }
+    quads[i].pair[0] = pair_rec(d[0], d[1]);
+    quads[i].pair[1] = pair_rec(d[2], d[3]);
+    tails[i] = t;
 }
 
 __global__ void k_update_emission(int64_t n, const uint32_t* __restrict__ perm, const float* __restrict__ emis,
@@ -622,7 +632,8 @@ int build_tree(rll_ctx* ctx, const float* tri, const float* emission, int64_t n,
     RLL_ALLOC(t->nodes, sizeof(NodeRec) * nn);
     RLL_ALLOC(t->pairs, sizeof(PairRec) * (n - 1));
     RLL_ALLOC(t->tails, sizeof(PairTail) * (n - 1));
-    RLL_ALLOC(t->quads, sizeof(DescRec) * 4 * (n - 1));
+    RLL_ALLOC(t->quads, sizeof(QuadRec) * (n - 1));
+    RLL_ALLOC(t->quad_tails, sizeof(QuadTail) * (n - 1));
     RLL_ALLOC(t->lights, sizeof(LightRec) * n);
     RLL_ALLOC(t->perm, sizeof(uint32_t) * n);
     RLL_ALLOC(t->left, sizeof(int32_t) * (n - 1));
@@ -630,15 +641,18 @@ int build_tree(rll_ctx* ctx, const float* tri, const float* emission, int64_t n,
     RLL_ALLOC(t->parent, sizeof(int32_t) * nn);
     RLL_ALLOC(t->light_cdf, sizeof(float) * n);
 #undef RLL_ALLOC
-    if (n > 1) {
+    if (n > 1) {  // powers and ids as texels
         cudaResourceDesc res{};
         res.resType = cudaResourceTypeLinear;
-        res.res.linear.devPtr = t->tails;
         res.res.linear.desc = cudaCreateChannelDesc<float4>();
-        res.res.linear.sizeInBytes = sizeof(PairTail) * (size_t)(n - 1);
         cudaTextureDesc tex{};
         tex.readMode = cudaReadModeElementType;
+        res.res.linear.devPtr = t->tails;
+        res.res.linear.sizeInBytes = sizeof(PairTail) * (size_t)(n - 1);
         e = cudaCreateTextureObject(&t->tail_tex, &res, &tex, nullptr);
+        res.res.linear.devPtr = t->quad_tails;
+        res.res.linear.sizeInBytes = sizeof(QuadTail) * (size_t)(n - 1);
+        if (e == cudaSuccess) e = cudaCreateTextureObject(&t->quad_tex, &res, &tex, nullptr);
         if (e != cudaSuccess) return check_cuda(ctx, e, "texture (tree)");
     }
     // scratch: codes, idx, sort, begin/end (unused after build), axis sums,
@@ -712,7 +726,7 @@ int build_tree(rll_ctx* ctx, const float* tri, const float* emission, int64_t n,
     k_finalize<<<grid_for(nn), kBlock, 0, s>>>(nn, t->nodes, cosmin);
     k_pairs<<<grid_for(n), kBlock, 0, s>>>(n, t->nodes, t->left, t->right, t->pairs, t->tails,
                                         leaf_phi);
-    if (n > 1) k_quads<<<grid_for(n - 1), kBlock, 0, s>>>(n, t->nodes, t->left, t->right, t->quads);
+    if (n > 1) k_quads<<<grid_for(n - 1), kBlock, 0, s>>>(n, t->nodes, t->left, t->right, t->quads, t->quad_tails);
     e = inclusive_scan_f32(s, leaf_phi, t->light_cdf, n, scan_ws);
     if (e != cudaSuccess) return check_cuda(ctx, e, "scan (light cdf)");
     e = cudaGetLastError();
