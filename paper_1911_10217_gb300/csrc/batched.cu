@@ -103,7 +103,7 @@ __global__ void __launch_bounds__(256) k_item_box_tables(const BatchItemDev* __r
     const int it = blockIdx.x;
     if (it >= n_items) return;
     const SampleArgs& a = items[it].s;
-    if (a.n_boxes > 0) build_box_table(a.boxes, a.n_boxes, static_cast<char*>(const_cast<void*>(a.box_table)));
+    if (a.n_boxes > 0) build_box_table_global(a.boxes, a.n_boxes, static_cast<char*>(const_cast<void*>(a.box_table)));
 }
 
 __device__ __forceinline__ int item_of_cell(const uint32_t* __restrict__ cell_prefix, int n_items, uint32_t cell)
@@ -321,8 +321,7 @@ cudaError_t launch_sample(rll_batch* b, cudaStream_t s)
 template <int P>
 cudaError_t launch_learn_t(rll_batch* b, cudaStream_t s, bool do_split)
 {
-    cudaError_t e = cudaMemsetAsync(b->n_touched, 0, 8 * sizeof(uint32_t), s);
-    if (e != cudaSuccess || b->n_records == 0) return e;
+    if (b->n_records == 0) return cudaMemsetAsync(b->n_touched, 0, 8 * sizeof(uint32_t), s);
     const int sms = device_sm_count(b->device);
     const BatchDec dec{b->total_cells << kBatchClusterBits};
     const BatchRows<P> rows{b->d_items, b->n, b->d_cell_prefix};

@@ -12,8 +12,9 @@
 // (NaN) takes the bin that keeps every box.
 //
 // The table is rebuilt from the boxes by one block before every launch that
-// reads it (3 us; the boxes may change from call to call) and copied to
-// shared memory by each block that does.
+// reads it (3.8 us; the boxes may change from call to call) and copied to
+// shared memory by each block that does. A sampling launch of few blocks and
+// boxes is done without: each block builds the table for itself (sample.cu).
 // Against one run of the boxes sorted along x, which every segment searched
 // and then walked through (and, in the energy sampler and the bounces, against
 // every box): 12-scene batch equal, 1080p passes 424 -> 416 us, sky dome (128
@@ -26,6 +27,7 @@
 #include "rll_device.cuh"
 
 namespace rll {
+namespace {  // build_box_table is out of line: every translation unit has its own copy
 
 // Bins an axis, and 64-bit words a mask, for n boxes: the table is 1.5 KB at 64 boxes, 6 KB at 256
 // and 12 KB at 1024 (where half as many bins keep it and the boxes within 48 KB).
@@ -86,13 +88,12 @@ struct BoxTable {
     }
 };
 
-// Builds the table of n (1 .. kMaxBoxes) boxes [n][6] into out, by a whole block of 256 threads.
-__device__ __forceinline__ void build_box_table(const float* __restrict__ boxes, int n, char* __restrict__ out)
+// Builds the table of n (1 .. kMaxBoxes) boxes [n][6] into out, by a whole block of at most 256
+// threads; s_mask: its masks in shared memory, or a scratch copy of them there (box_mask_bytes).
+__device__ __noinline__ void build_box_table(const float* __restrict__ boxes, int n, char* out, uint32_t* s_mask)
 {
-    __shared__ uint32_t s_mask[box_mask_bytes(kMaxBoxes) / 4];
     __shared__ float s_lim[8][6];
     __shared__ float s_scale[3], s_off[3];
-    static_assert(box_mask_bytes(kMaxBoxes) >= box_mask_bytes(256), "largest table");
     const int bins = box_bins(n), words = 2 * box_words(n), lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     for (int i = threadIdx.x; i < 6 * bins * words; i += blockDim.x) s_mask[i] = 0u;
     float lim[6] = {INFINITY, INFINITY, INFINITY, -INFINITY, -INFINITY, -INFINITY};
@@ -153,12 +154,28 @@ __device__ __forceinline__ void build_box_table(const float* __restrict__ boxes,
     }
     __syncthreads();
     uint32_t* mask = reinterpret_cast<uint32_t*>(out + 32);
-    for (int i = threadIdx.x; i < 6 * bins * words; i += blockDim.x) mask[i] = s_mask[i];
+    if (mask != s_mask)
+        for (int i = threadIdx.x; i < 6 * bins * words; i += blockDim.x) mask[i] = s_mask[i];
+}
+
+// The same by a block that writes the table to global memory.
+__device__ __forceinline__ void build_box_table_global(const float* __restrict__ boxes, int n, char* out)
+{
+    __shared__ uint32_t s_mask[box_mask_bytes(kMaxBoxes) / 4];
+    static_assert(box_mask_bytes(kMaxBoxes) >= box_mask_bytes(256), "largest table");
+    build_box_table(boxes, n, out, s_mask);
 }
 
 // The table copied to shared memory by all threads of the block (the caller synchronises).
-__device__ __forceinline__ BoxTable stage_box_table(void* s_table, const void* table, int n)
+// SELF: without a table (nullptr) the block builds its own from the boxes.
+template <bool SELF = false>
+__device__ __forceinline__ BoxTable stage_box_table(void* s_table, const void* table, int n,
+                                                    const float* boxes = nullptr)
 {
+    if (SELF && !table && n > 0) {
+        build_box_table(boxes, n, static_cast<char*>(s_table), reinterpret_cast<uint32_t*>(s_table) + 8);
+        return BoxTable{static_cast<const char*>(s_table), n};
+    }
     const float4* src = static_cast<const float4*>(table);
     float4* dst = static_cast<float4*>(s_table);
     if (n > 0)
@@ -166,4 +183,5 @@ __device__ __forceinline__ BoxTable stage_box_table(void* s_table, const void* t
     return BoxTable{static_cast<const char*>(s_table), n};
 }
 
+}  // namespace
 }  // namespace rll

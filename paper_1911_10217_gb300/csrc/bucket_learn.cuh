@@ -106,20 +106,17 @@ k_bucket_count(const uint32_t* __restrict__ rec_key, int64_t n, Dec dec, uint32_
         if (old[u] == 0u) touched[base++] = slot[u];
 }
 
-// 2. one contiguous bucket per touched cell (one atomic per warp)
-__global__ void __launch_bounds__(kBucketThreads)
-k_bucket_claim(const uint32_t* __restrict__ touched, uint32_t* __restrict__ ctr, uint32_t* __restrict__ cursor,
-               uint32_t* __restrict__ start, uint32_t* __restrict__ len, uint32_t* __restrict__ group_list,
-               uint32_t* __restrict__ sort_list, uint32_t cells)
+// 2. one contiguous bucket per touched cell (one atomic per warp), by `warps` warps of which this is
+// number `first`
+__device__ __forceinline__ void claim_cells(uint32_t first, uint32_t warps, uint32_t total, const uint32_t* touched,
+                                            uint32_t* ctr, uint32_t* cursor, uint32_t* start, uint32_t* len,
+                                            uint32_t* group_list, uint32_t* sort_list, uint32_t cells)
 {
-    pdl_begin();
-    const uint32_t total = *(volatile uint32_t*)ctr;
     const int lane = threadIdx.x & 31;
-    const uint32_t warps = gridDim.x * (blockDim.x >> 5);
-    for (uint32_t w = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); w * 32 < total; w += warps) {
+    for (uint32_t w = first; w * 32 < total; w += warps) {
         const uint32_t c = w * 32 + lane;
-        const uint32_t slot = c < total ? touched[c] : 0u;
-        const uint32_t cnt = c < total ? cursor[slot] : 0u;
+        const uint32_t slot = c < total ? __ldcg(touched + c) : 0u;
+        const uint32_t cnt = c < total ? __ldcg(cursor + slot) : 0u;
         uint32_t x = cnt;
 #pragma unroll
         for (int o = 1; o < 32; o <<= 1) {
@@ -153,6 +150,16 @@ k_bucket_claim(const uint32_t* __restrict__ touched, uint32_t* __restrict__ ctr,
         if (to_group) group_list[cells - 1u - (gb + __popc(gm & below))] = c;
         if (to_sort) sort_list[sb + __popc(sm & below)] = c;
     }
+}
+
+__global__ void __launch_bounds__(kBucketThreads)
+k_bucket_claim(const uint32_t* __restrict__ touched, uint32_t* __restrict__ ctr, uint32_t* __restrict__ cursor,
+               uint32_t* __restrict__ start, uint32_t* __restrict__ len, uint32_t* __restrict__ group_list,
+               uint32_t* __restrict__ sort_list, uint32_t cells)
+{
+    pdl_begin();
+    claim_cells(blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5), gridDim.x * (blockDim.x >> 5),
+                *(volatile uint32_t*)ctr, touched, ctr, cursor, start, len, group_list, sort_list, cells);
 }
 
 // 3. every record to its cell's bucket, at the bucket start (the claim left it
@@ -209,6 +216,78 @@ k_bucket_scatter(const uint32_t* __restrict__ rec_key, const float* __restrict__
     for (int u = 0; u < kTilesPerWarp; ++u) {
         if (!dec.valid(key[u])) continue;
         bucket.put(at[u] + rk[u], (uint32_t)(i0 + (int64_t)u * kBucketThreads), dec.cluster(key[u]), val[u]);
+    }
+}
+
+// 1. to 3. for few records in one launch: one cluster of blocks, its barrier between the steps, the
+// counters cleared and the ranks kept in registers. The three launches, a clearing and the gaps
+// between them took longer than the work (16 384 records, 64x64 points: 44.5 -> 42 us a pass; 12 288,
+// 48.3 -> 46.5; with four times as many records a thread, 30 000 records: 52.9 -> 55.7); above
+// kSmallRecords more SMs than a cluster's are worth more than the launches.
+constexpr int kSmallBlocks = 8, kSmallThreads = 1024, kSmallItems = 2;
+constexpr int64_t kSmallRecords = (int64_t)kSmallBlocks * kSmallThreads * kSmallItems;
+
+__device__ __forceinline__ void cluster_sync()
+{
+    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+
+template <class Dec>
+__global__ void __cluster_dims__(kSmallBlocks, 1, 1) __launch_bounds__(kSmallThreads)
+k_bucket_small(const uint32_t* __restrict__ rec_key, const float* __restrict__ rec_val, uint32_t n, Dec dec,
+               uint32_t* cursor, uint32_t* touched, uint32_t* ctr, uint32_t* start, uint32_t* len,
+               uint32_t* group_list, uint32_t* sort_list, uint32_t cells, Bucket bucket)
+{
+    pdl_wait();
+    const uint32_t lane = threadIdx.x & 31u, g = blockIdx.x * kSmallThreads + threadIdx.x;
+    if (g < 8) ctr[g] = 0u;
+    __threadfence();
+    cluster_sync();
+    uint32_t key[kSmallItems], rank[kSmallItems];
+#pragma unroll
+    for (int u = 0; u < kSmallItems; ++u) {
+        const uint32_t i = (uint32_t)u * (kSmallBlocks * kSmallThreads) + g;
+        key[u] = i < n ? __ldg(rec_key + i) : 0xFFFFFFFFu;
+    }
+    uint32_t peers[kSmallItems];
+#pragma unroll
+    for (int u = 0; u < kSmallItems; ++u)
+        peers[u] = __match_any_sync(0xffffffffu, dec.valid(key[u]) ? dec.cell(key[u]) : 0xFFFFFFFFu);
+#pragma unroll
+    for (int u = 0; u < kSmallItems; ++u) {
+        rank[u] = 1u;
+        if (dec.valid(key[u]) && lane == (uint32_t)(__ffs(peers[u]) - 1))
+            rank[u] = atomicAdd(cursor + dec.cell(key[u]), (uint32_t)__popc(peers[u]));
+    }
+    uint32_t fresh = 0;
+#pragma unroll
+    for (int u = 0; u < kSmallItems; ++u) fresh |= (rank[u] == 0u) << u;
+    uint32_t x = __popc(fresh);
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t y = __shfl_up_sync(0xffffffffu, x, o);
+        if (lane >= o) x += y;
+    }
+    uint32_t at = 0;
+    if (lane == 31 && x) at = atomicAdd(ctr, x);
+    at = __shfl_sync(0xffffffffu, at, 31) + x - __popc(fresh);
+#pragma unroll
+    for (int u = 0; u < kSmallItems; ++u) {
+        if (fresh >> u & 1u) touched[at++] = dec.cell(key[u]);
+        rank[u] = __shfl_sync(0xffffffffu, rank[u], __ffs(peers[u]) - 1) + __popc(peers[u] & lanemask_lt());
+    }
+    __threadfence();
+    cluster_sync();
+    claim_cells(g >> 5, kSmallBlocks * kSmallThreads / 32, *(volatile uint32_t*)ctr, touched, ctr, cursor, start, len,
+                group_list, sort_list, cells);
+    __threadfence();
+    cluster_sync();
+    pdl_release();  // the next kernel reads the counts as soon as it starts
+#pragma unroll
+    for (int u = 0; u < kSmallItems; ++u) {
+        const uint32_t i = (uint32_t)u * (kSmallBlocks * kSmallThreads) + g;
+        if (!dec.valid(key[u])) continue;
+        bucket.put(__ldcg(cursor + dec.cell(key[u])) + rank[u], i, dec.cluster(key[u]), __float_as_uint(__ldg(rec_val + i)));
     }
 }
 
@@ -489,7 +568,9 @@ __device__ void compose_sorted_block(Cls cls, Val val, uint32_t nr, uint32_t M, 
 // (more than kPairBucket records; the ordering of the warp path done by the
 // whole block, warps composing different clusters in parallel). Phase 1: the
 // block's warp pairs take the cells of the two-warp list (kWarpBucket ..
-// kPairBucket records), three cells per block at a time. Phase 2: warps take
+// kPairBucket records), three cells per block at a time; where there are no
+// more such cells than blocks, blocks take them in phase 0 (64-sample tile:
+// 305 us a pass, now 295). Phase 2: warps take
 // the touched cells one by one and order those of at most kWarpBucket records
 // themselves. Every phase draws from an atomic work counter (ctr[4], ctr[7],
 // ctr[5]), so the long cells start first and the teams that drew one join the
@@ -517,7 +598,8 @@ k_learn_buckets(const Bucket bucket, uint32_t* __restrict__ ctr, const uint32_t*
     // complete and visible (each block waits for it first), and ends only when k_learn_big has, so
     // that whatever follows this kernel follows both. Where it has none, k_learn_big releases this
     // kernel at once and ends with the scatter, for which this kernel's blocks wait in their places.
-    // (The claim, which writes the counts, is complete before any block of the scatter releases.)
+    // (The claim, which writes the counts, is complete before any block of the scatter, or of
+    // k_bucket_small, releases.)
     const bool beside = *(volatile const uint32_t*)(ctr + 2) != 0u;
     if (!beside) pdl_wait();
     pdl_release();
@@ -527,8 +609,13 @@ k_learn_buckets(const Bucket bucket, uint32_t* __restrict__ ctr, const uint32_t*
     __shared__ __align__(16) unsigned char smem[WARPS * L::kSlab];
     __shared__ uint32_t s_next, s_pair[WARPS / 2];
     const uint32_t warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const uint32_t n_group = *(volatile const uint32_t*)(ctr + 6);
-    const uint32_t n_pair = *(volatile const uint32_t*)(ctr + 3);
+    const uint32_t n_block_list = *(volatile const uint32_t*)(ctr + 6);
+    uint32_t n_pair = *(volatile const uint32_t*)(ctr + 3);
+    uint32_t n_group = n_block_list;
+    if (n_group + n_pair <= gridDim.x) {  // a block for each of them: the pairs' cells too
+        n_group += n_pair;
+        n_pair = 0;
+    }
     const uint32_t total = *(volatile const uint32_t*)ctr;
     uint32_t phase = n_group ? 0u : (n_pair ? 1u : 2u), ahead = 0;
     bool drawn = false;  // phase 2: `ahead` holds the next index
@@ -544,7 +631,7 @@ k_learn_buckets(const Bucket bucket, uint32_t* __restrict__ ctr, const uint32_t*
                 phase = 1;
                 continue;
             }
-            w = group_list[cells - 1u - bi];
+            w = group_list[bi < n_block_list ? cells - 1u - bi : bi - n_block_list];
             team = Team{threadIdx.x, (uint32_t)(WARPS * 32)};
         } else if (phase == 1) {
             team = Team{threadIdx.x & 63u, 64u};
@@ -807,8 +894,8 @@ inline size_t bucketed_scratch_bytes(int64_t n)
 
 // Enqueues the whole learning step for n >= 1 records (cut sizes up to
 // max_cut), every kernel with the programmatic launch dependency (each waits
-// for its predecessor first). The caller has zeroed ctr[0..7] on the stream
-// and holds `cursor` [cells] at zero (left at zero again); touched, start,
+// for its predecessor first). Clears ctr[0..7] first; the caller holds
+// `cursor` [cells] at zero (left at zero again); touched, start,
 // len [cells] and lists [2 * cells] are outputs and scratch. Counters: ctr[0]
 // touched cells, [1] claimed records, [2] sorting list, [3] two-warp list,
 // [6] block list, [4] [5] [7] work counters of k_learn_buckets.
@@ -832,14 +919,22 @@ cudaError_t launch_bucketed_learn(cudaStream_t s, int device, int sms, const uin
     uint32_t* sort_list = lists + cells;
     // record ranks: the first 4 n bytes of the in-place sort buffer (dead until k_learn_big)
     uint32_t* rank = reinterpret_cast<uint32_t*>(wide);
-    cudaError_t e0 = launch_pdl(k_bucket_count<Dec>, dim3(rblocks), dim3(kBucketThreads), 0, s, rec_key, n, dec,
-                                cursor, touched, ctr, rank);
-    if (e0 == cudaSuccess)
-        e0 = launch_pdl(k_bucket_claim, dim3(sms * 2), dim3(kBucketThreads), 0, s, touched, ctr, cursor, start, len,
-                        group_list, sort_list, cells);
-    if (e0 == cudaSuccess)
-        e0 = launch_pdl(k_bucket_scatter<Dec>, dim3(rblocks), dim3(kBucketThreads), 0, s, rec_key, rec_val, n, dec,
-                        cursor, rank, bucket);
+    cudaError_t e0;
+    if (n <= kSmallRecords) {
+        e0 = launch_pdl(k_bucket_small<Dec>, dim3(kSmallBlocks), dim3(kSmallThreads), 0, s, rec_key, rec_val, (uint32_t)n,
+                        dec, cursor, touched, ctr, start, len, group_list, sort_list, cells, bucket);
+    } else {
+        e0 = cudaMemsetAsync(ctr, 0, 8 * sizeof(uint32_t), s);
+        if (e0 == cudaSuccess)
+            e0 = launch_pdl(k_bucket_count<Dec>, dim3(rblocks), dim3(kBucketThreads), 0, s, rec_key, n, dec, cursor,
+                            touched, ctr, rank);
+        if (e0 == cudaSuccess)
+            e0 = launch_pdl(k_bucket_claim, dim3(sms * 2), dim3(kBucketThreads), 0, s, touched, ctr, cursor, start,
+                            len, group_list, sort_list, cells);
+        if (e0 == cudaSuccess)
+            e0 = launch_pdl(k_bucket_scatter<Dec>, dim3(rblocks), dim3(kBucketThreads), 0, s, rec_key, rec_val, n, dec,
+                            cursor, rank, bucket);
+    }
     if (e0 != cudaSuccess) return e0;
     // k_learn_big first, k_learn_buckets beside it: its blocks, few and long, take the place they need,
     // and without cells for them they cost nothing (whole passes: 64-sample tile 346 -> 307 us, path

@@ -271,17 +271,20 @@ template <int P, class Split = NoSplit>
 int learn_t(rll_ctx* ctx, rll_grid* g, const uint32_t* rec_key, const float* rec_val, int64_t n, Split sp = Split{})
 {
     cudaStream_t s = ctx->stream;
-    cudaError_t e = cudaMemsetAsync(g->n_touched, 0, 8 * sizeof(uint32_t), s);
-    if (e != cudaSuccess) return check_cuda(ctx, e, "memset touched");
-    if (n <= 0) return RLL_OK;
-    if (n > 0xFFFFFFFFll) return fail(ctx, RLL_E_INVALID, "more than 2^32 - 1 records");
+    cudaError_t e = cudaSuccess;
+    void* ws = n > 0 && n <= 0xFFFFFFFFll ? ws_get(ctx, bucketed_scratch_bytes(n)) : nullptr;
+    if (!ws) {  // no touched cells (otherwise the learning kernels clear the count)
+        e = cudaMemsetAsync(g->n_touched, 0, 8 * sizeof(uint32_t), s);
+        if (e != cudaSuccess) return check_cuda(ctx, e, "memset touched");
+        if (n <= 0) return RLL_OK;
+        if (n > 0xFFFFFFFFll) return fail(ctx, RLL_E_INVALID, "more than 2^32 - 1 records");
+        return RLL_E_NOMEM;
+    }
     if (g->cursor_dirty) {
         e = cudaMemsetAsync(g->cursor, 0, 4 * (size_t)g->H, s);
         if (e != cudaSuccess) return check_cuda(ctx, e, "memset cursors");
         g->cursor_dirty = false;
     }
-    void* ws = ws_get(ctx, bucketed_scratch_bytes(n));
-    if (!ws) return RLL_E_NOMEM;
     using T = typename Store<P>::T;
     g->cursor_dirty = true;
     e = launch_bucketed_learn<P>(s, g->device, device_sm_count(g->device), rec_key, rec_val, n,

@@ -40,7 +40,7 @@ __global__ void __launch_bounds__(THREADS, MINB) k_sample(SampleArgs a)
 {
     pdl_begin();
     extern __shared__ float4 s_boxes[];
-    const BoxTable bt = stage_box_table(s_boxes, a.box_table, a.n_boxes);
+    const BoxTable bt = stage_box_table<SPLIT != LOOP>(s_boxes, a.box_table, a.n_boxes, a.boxes);
     if constexpr (SPLIT == LANES) {
         __shared__ float s_est[THREADS / 32][kWarpEst];
         __syncthreads();
@@ -109,7 +109,7 @@ __global__ void __launch_bounds__(kThreads) k_sample_power(SampleArgs a, int32_t
 __global__ void __launch_bounds__(256) k_box_table(const float* __restrict__ boxes, int n, char* __restrict__ out)
 {
     pdl_begin();
-    build_box_table(boxes, n, out);
+    build_box_table_global(boxes, n, out);
 }
 
 template <int P, int MODE, bool DBG, int SPLIT, int THREADS, int MINB>
@@ -147,8 +147,15 @@ int sample_and_shade(rll_ctx* ctx, rll_grid* g, const rll_tree* t, const float* 
                      uint32_t frame, int spp, float* rgb, uint32_t* rec_key, float* rec_val,
                      const rll_sample_debug* dbg)
 {
+    // Up to 64 boxes and one wave of blocks: each block builds the boxes' table for itself, about as
+    // long as a block alone takes, but without a launch (64x64 points: 42 -> 39 us a pass). In larger
+    // launches the copies would cost more than one build.
+    const uint32_t warp_points = lane_split(n_points, spp, 32 * (int64_t)device_sm_count(ctx->device));
+    const int64_t warps = warp_points ? (n_points + warp_points - 1) / warp_points : (n_points + 31) / 32;
+    const bool loop = (spp > 1 && !warp_points) || (dbg && (dbg->light || dbg->p_cut || dbg->p_in));
+    const bool self = !loop && n_boxes <= 64 && warps <= 32 * (int64_t)device_sm_count(ctx->device);
     const void* table = nullptr;
-    const int rc = box_table(ctx, boxes, n_boxes, ctx->stream, &table);
+    const int rc = self ? RLL_OK : box_table(ctx, boxes, n_boxes, ctx->stream, &table);
     if (rc != RLL_OK) return rc;
     return sample_and_shade_range(ctx, g, t, pos, nrm, albedo, footprint, n_points, 0, n_points, boxes, n_boxes, seed,
                                   frame, spp, rgb, rec_key, rec_val, dbg, ctx->stream, table);

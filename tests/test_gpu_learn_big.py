@@ -48,3 +48,32 @@ def test_eq1_in_large_cells(env, counts, length, skew):  # noqa: F811
     # a composed value carries at most some 40 roundings (2^-24 each) of the last records' weight
     assert np.allclose(q[: len(counts), :m], want[: len(counts), :m], rtol=1e-5, atol=0.0)
     assert np.array_equal(q[len(counts):], q0[len(counts):])
+
+
+@pytest.mark.parametrize("records", [1, 31, 8191, 8193, 16384, 16385])
+def test_bucketing_sizes(env, records):  # noqa: F811
+    """Up to 16 384 records are bucketed by one cluster of blocks, more by three launches: record
+    counts around a round of the cluster (8 192) and its last, twice in a row from the same grid."""
+    import torch
+    rll, ctx, dev = env["rll"], env["ctx"], env["dev"]
+    ctx.sync_status()
+    s = scenes.tiny_scene()
+    d = device_scene(s, dev)
+    alpha = 0.25
+    tree = rll.Tree(ctx, d["tri"], d["em"])
+    grid = rll.Grid(ctx, tree, params_for(rll, s, alpha=alpha))
+    M, m = grid.M, grid.m
+    rng = np.random.default_rng(records)
+    want = grid.export()["q"].astype(np.float64)
+    for turn in range(2):
+        key = rng.integers(0, 300, records) * M + rng.integers(0, m, records)
+        bad = rng.uniform(size=records) < 0.05
+        val = rng.uniform(0.1, 2.0, records).astype(np.float32)
+        rll.learn_update(ctx, grid, torch.from_numpy(np.where(bad, -1, key).astype(np.int32)).to(dev),
+                         torch.from_numpy(val).to(dev))
+        for k, v in zip(key[~bad], val[~bad].astype(np.float64)):
+            want[k // M, k % M] = (1.0 - alpha) * want[k // M, k % M] + alpha * v
+        assert ctx.sync_status() == 0 and grid.touched_cells() == np.unique(key[~bad] // M).size
+        q = grid.export()["q"]
+        # some 40 roundings of 2^-24 a turn, see above
+        assert np.allclose(q[:, :m], want[:, :m], rtol=2e-5, atol=0.0)
