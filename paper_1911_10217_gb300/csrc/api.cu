@@ -10,6 +10,7 @@
 #include <string>
 #include <vector>
 
+#include "box_bins.cuh"
 #include "rll_device.cuh"
 #include "rll_internal.h"
 
@@ -175,8 +176,11 @@ int rll_ctx_create(rll_ctx** out, int device, void* cuda_stream)
     ctx->stream = (cudaStream_t)cuda_stream;
     DeviceGuard g(device);
     if (cudaMalloc(&ctx->d_status, sizeof(uint32_t)) != cudaSuccess ||
+        cudaMalloc(&ctx->box_table, kMaxBoxTable) != cudaSuccess ||
         cudaMemset(ctx->d_status, 0, sizeof(uint32_t)) != cudaSuccess) {
         cudaGetLastError();
+        cudaFree(ctx->d_status);
+        cudaFree(ctx->box_table);
         delete ctx;
         return RLL_E_NOMEM;
     }

@@ -572,7 +572,7 @@ __device__ void compose_sorted_block(Cls cls, Val val, uint32_t nr, uint32_t M, 
 // more such cells than blocks, blocks take them in phase 0 (64-sample tile:
 // 305 us a pass, now 295). Phase 2: warps take
 // the touched cells one by one and order those of at most kWarpBucket records
-// themselves. Every phase draws from an atomic work counter (ctr[4], ctr[7],
+// themselves. Every phase draws from a work counter (ctr[4], ctr[7],
 // ctr[5]), so the long cells start first and the teams that drew one join the
 // next phase late instead of leaving a tail; a warp fetches its next cell
 // index while it works on the current one. Shared memory: one slab per warp;
@@ -617,44 +617,72 @@ k_learn_buckets(const Bucket bucket, uint32_t* __restrict__ ctr, const uint32_t*
         n_pair = 0;
     }
     const uint32_t total = *(volatile const uint32_t*)ctr;
-    uint32_t phase = n_group ? 0u : (n_pair ? 1u : 2u), ahead = 0;
-    bool drawn = false;  // phase 2: `ahead` holds the next index
+    uint32_t phase = n_group ? 0u : (n_pair ? 1u : 2u);
+    // A team's first cell is its own number; only then does it draw from the phase's counter, whose
+    // values follow the teams' numbers. Warps draw several cells at a time, an eighth of their share of
+    // those left but at most 8: all the warps' draws of single cells from one address, one after another in the
+    // L2, held a warp back for 5 000 cycles of the 17 000 that it spent on a cell (1080p; 12 000 of
+    // 21 000 with two cells a warp). Passes: 64x64 points 40.5 -> 33.7 us, preview 80 -> 76, 1080p
+    // 384 -> 378, 4K 1 843 -> 1 835 (with a quarter of the share at once 1 865: a tail).
+    const uint32_t teams = gridDim.x * WARPS;
+    auto share = [&](uint32_t left) { return min(max(left / (8 * teams), 1u), 8u); };
+    const uint32_t chunk0 = share(total);
+    bool first = true;              // of the phase
+    uint32_t next = 0, end = 0;     // phase 2: the warp's cells
+    uint32_t ahead = 0, len_ahead = 0;  // its next draw, `ahead` on lane 0
     for (;;) {
         uint32_t w;  // index of the next cell in the touched list
         Team team;
         if (phase == 0) {
-            if (threadIdx.x == 0) s_next = atomicAdd(ctr + 4, 1u);
-            __syncthreads();
-            const uint32_t bi = s_next;
-            __syncthreads();
-            if (bi >= n_group) {  // uniform across the block: every warp leaves phase 0
+            uint32_t bi = blockIdx.x;
+            if (!first && n_group > gridDim.x) {
+                if (threadIdx.x == 0) s_next = gridDim.x + atomicAdd(ctr + 4, 1u);
+                __syncthreads();
+                bi = s_next;
+                __syncthreads();
+            }
+            if (bi >= n_group || (!first && n_group <= gridDim.x)) {  // uniform across the block: it leaves phase 0
                 phase = 1;
+                first = true;
                 continue;
             }
+            first = false;
             w = group_list[bi < n_block_list ? cells - 1u - bi : bi - n_block_list];
             team = Team{threadIdx.x, (uint32_t)(WARPS * 32)};
         } else if (phase == 1) {
+            const uint32_t pairs = gridDim.x * (WARPS / 2);
             team = Team{threadIdx.x & 63u, 64u};
-            if (team.tid == 0) s_pair[warp >> 1] = atomicAdd(ctr + 7, 1u);
-            team.sync();
-            const uint32_t pi = s_pair[warp >> 1];
-            team.sync();
-            if (pi >= n_pair) {  // uniform across the pair: the shared memory is per warp now
+            uint32_t pi = blockIdx.x * (WARPS / 2) + (warp >> 1);
+            if (!first && n_pair > pairs) {
+                if (team.tid == 0) s_pair[warp >> 1] = pairs + atomicAdd(ctr + 7, 1u);
+                team.sync();
+                pi = s_pair[warp >> 1];
+                team.sync();
+            }
+            if (pi >= n_pair || (!first && n_pair <= pairs)) {  // uniform across the pair: it leaves phase 1
                 phase = 2;
+                first = true;
                 continue;
             }
+            first = false;
             w = group_list[pi];
         } else {
             team = Team{lane, 32u};
-            if (!drawn && lane == 0) ahead = atomicAdd(ctr + 5, 1u);
-            w = __shfl_sync(0xffffffffu, ahead, 0);
-            if (w >= total) break;
-            if (lane == 0) ahead = atomicAdd(ctr + 5, 1u);
-            drawn = true;
+            if (first || next == end) {
+                const uint32_t count = first ? chunk0 : len_ahead;
+                if (first) next = (blockIdx.x * WARPS + warp) * chunk0;
+                else next = teams * chunk0 + __shfl_sync(0xffffffffu, ahead, 0);
+                first = false;
+                if (next >= total) break;
+                end = min(next + count, total);
+                len_ahead = share(total - next);
+                ahead = total;
+                if (lane == 0 && teams * chunk0 < total) ahead = atomicAdd(ctr + 5, len_ahead);
+            }
+            w = next++;
         }
-        const uint32_t slot = touched[w], nr = len[w];
+        const uint32_t slot = touched[w], nr = len[w], b0 = start[w];
         if (phase == 2 && nr > kWarpBucket) continue;
-        const uint32_t b0 = start[w];
         const RowRef<P> r = rows.row(slot);
         const uint32_t slab = phase == 0 ? 0u : (phase == 1 ? warp & ~1u : warp);
         const uint32_t cap = phase == 0 ? kBlockGroup : (phase == 1 ? kPairBucket : kWarpBucket);

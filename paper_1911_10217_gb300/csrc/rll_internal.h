@@ -40,8 +40,8 @@ struct rll_ctx {
     int host_zero_copy = 1;  // rll_render_pass_host: use mapped host buffers in place
     // launch tuning (rll_ctx_set_option)
     int sample_min_blocks = 4;
-    // the occluder boxes' table (box_bins.cuh), rebuilt by every call that reads boxes (sample.cu:
-    // box_table); allocated on first use
+    // the occluder boxes' table (box_bins.cuh), rebuilt by the calls that read boxes (sample.cu:
+    // box_table)
     void* box_table = nullptr;
 };
 

@@ -165,13 +165,6 @@ int box_table(rll_ctx* ctx, const float* boxes, int n_boxes, cudaStream_t stream
 {
     *out = nullptr;
     if (n_boxes <= 0) return RLL_OK;
-    if (!ctx->box_table) {
-        if (cudaMalloc(&ctx->box_table, kMaxBoxTable) != cudaSuccess) {
-            cudaGetLastError();
-            ctx->box_table = nullptr;
-            return fail(ctx, RLL_E_NOMEM, "cannot allocate the box table");
-        }
-    }
     const int rc = check_cuda(ctx,
                               launch_pdl(k_box_table, dim3(1), dim3(256), 0, stream, boxes, n_boxes,
                                          static_cast<char*>(ctx->box_table)),
