@@ -63,12 +63,29 @@ __global__ void __launch_bounds__(THREADS, MINB) k_sample(SampleArgs a)
     }
 }
 
-// Energy-based baseline (Section 4): inversion of the cdf of leaf power.
+// Energy-based baseline (Section 4): inversion of the cdf of leaf power, by the binary search over all
+// lights whose first kPowerLevels probes, the same for every sample up to their outcomes, each block
+// keeps in shared memory as a heap (node h's children 2h, where the probe is above the draw, and 2h +
+// 1): probes of so long an array are gathers of one sector each (64K lights, 4 samples a point,
+// 1080p: 392 us, now 318).
+constexpr int kPowerLevels = 9;  // 2 KB beside the box table of up to 45 KB
+
 __global__ void __launch_bounds__(kThreads) k_sample_power(SampleArgs a, int32_t* light_out)
 {
     pdl_begin();
     extern __shared__ float4 s_boxes[];
+    __shared__ float s_probe[1 << kPowerLevels];
     const BoxTable bt = stage_box_table(s_boxes, a.box_table, a.n_boxes);
+    const uint32_t last = (uint32_t)a.n_lights - 1u;
+    for (uint32_t h = 1 + threadIdx.x; h < (1u << kPowerLevels); h += blockDim.x) {
+        uint32_t lo = 0, hi = last;
+        for (int b = 30 - __clz((int)h); b >= 0 && lo < hi; --b) {  // the way to h from the root
+            const uint32_t mid = (lo + hi) >> 1;
+            if (h >> b & 1u) lo = mid + 1;
+            else hi = mid;
+        }
+        s_probe[h] = a.light_cdf[(lo + hi) >> 1];  // unused where the search has ended
+    }
     __syncthreads();
     const int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (p >= a.n_points) return;
@@ -76,21 +93,27 @@ __global__ void __launch_bounds__(kThreads) k_sample_power(SampleArgs a, int32_t
     const float x0 = a.pos[p], x1 = a.pos[np + p], x2 = a.pos[2 * np + p];
     const float n0 = a.nrm[p], n1 = a.nrm[np + p], n2 = a.nrm[2 * np + p];
     const float alb = a.albedo[p];
-    const int64_t nl = a.n_lights;
-    const float total = a.light_cdf[nl - 1];
+    const float total = a.light_cdf[last];
     float acc0 = 0.0f, acc1 = 0.0f, acc2 = 0.0f;
     for (int j = 0; j < a.spp; ++j) {
         const uint32_t sid = (uint32_t)(p * a.spp + j);
         SampleStream rs;
         rs.init(a.seed, sid, a.frame);
         const float u = rs.draw(kDrawCut);
-        int64_t lo = 0, hi = nl - 1;
+        uint32_t lo = 0, hi = last, h = 1;
+        for (int l = 0; l < kPowerLevels && lo < hi; ++l) {
+            const uint32_t mid = (lo + hi) >> 1;
+            const bool above = __fmaf_rn(-u, total, s_probe[h]) > 0.0f;
+            h = 2 * h + !above;
+            if (above) hi = mid;
+            else lo = mid + 1;
+        }
         while (lo < hi) {
-            const int64_t mid = (lo + hi) >> 1;
+            const uint32_t mid = (lo + hi) >> 1;
             if (__fmaf_rn(-u, total, a.light_cdf[mid]) > 0.0f) hi = mid;
             else lo = mid + 1;
         }
-        const float pl = a.nodes[nl - 1 + lo].phi / total;
+        const float pl = a.nodes[last + lo].phi / total;
         const LightRec Lr = load_light(a.lights + lo);
         const ShadeOut o = shade(Lr, x0, x1, x2, n0, n1, n2, alb, pl, 1.0f, rs.draw(kDrawTriA), rs.draw(kDrawTriB),
                                  bt, 0);

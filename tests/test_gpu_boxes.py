@@ -50,3 +50,26 @@ def test_bounce_over_the_table(env, n, far):  # noqa: F811
     rll.bounce_vertices(ctx, t(pos), t(nrm), t(boxes), scenes.ROOM, 9, 2, 50.0, y, ny, f)
     for got, want in ((y, oy), (ny, on), (f, of)):
         assert np.array_equal(got.cpu().numpy(), np.asarray(want, np.float32))
+
+
+@pytest.mark.parametrize("lights,boxes", [(1, 64), (2, 64), (3, 0), (400, 65), (512, 64), (513, 256), (4096, 1024)])
+def test_energy_sampler_search(env, lights, boxes):  # noqa: F811
+    """The light search's first nine probes come from shared memory: fewer lights than they tell
+    apart, as many, and more. The chosen light is the first whose prefix exceeds the draw."""
+    import torch
+    O, rll, ctx, dev = env["O"], env["rll"], env["ctx"], env["dev"]
+    s = scenes.frame_scene(seed=3, width=64, height=32, n_patches=16, tris_per_patch=256, n_boxes=32)
+    tris, emission = s.tris[:lights], s.emission[:lights]
+    s = dataclasses.replace(s, tris=tris, emission=emission, boxes=random_boxes(boxes))
+    t = lambda a: torch.from_numpy(np.ascontiguousarray(a)).to(dev)  # noqa: E731
+    tree = rll.Tree(ctx, t(tris.reshape(-1, 9)), t(emission))
+    ot = O.Tree(tris, emission)
+    P, spp = s.n_points, 5
+    rgb, light = torch.empty(3, P, device=dev), torch.empty(P * spp, dtype=torch.int32, device=dev)
+    rll.sample_power(ctx, tree, t(s.pos), t(s.nrm), t(s.albedo), t(s.boxes), 3, 0, spp, rgb, light)
+    orgb, olight = O.sample_power(ot, O.scene_arrays(s), 3, 0, spp)
+    lg = light.cpu().numpy()
+    # the device's prefix sums are binary32: draws within their rounding of a boundary may differ
+    assert np.mean(lg != olight) < 1e-3 and np.abs(lg - olight).max() <= 1
+    same = np.all((lg == olight).reshape(P, spp), axis=1)
+    assert np.allclose(rgb.cpu().numpy()[:, same], orgb[:, same], rtol=1e-3, atol=1e-7)
