@@ -96,18 +96,14 @@ k_bounce(const float* __restrict__ pos, const float* __restrict__ nrm, int64_t n
             axis = k;
         }
     }
-    // The nearest box face in front of it. A box whose face is met at t < t_best meets the segment's
-    // bounding box from o to there; widened by a margin above the rounding errors of the slab planes
-    // and of the segment's end (a few ulps of the coordinates), it keeps every box that counts.
-    float lo[3], hi[3];
-    for (int k = 0; k < 3; ++k) {
-        const float end = fadd(o[k], fmul(t_best, d[k]));  // NaN (every box kept) if d = 0 and no wall is ahead
-        const float e = 1e-5f * (1.0f + fabsf(o[k]) + fabsf(end));
-        lo[k] = fsub(end < o[k] ? end : o[k], e);
-        hi[k] = fadd(end > o[k] ? end : o[k], e);
-    }
+    // The nearest box face in front of it, in up to four segments of the ray, the first an eighth of
+    // the boxes' extent long, each other twice the one before and the last the rest: most rays end in
+    // the first two, near which few boxes are (path vertices at 720p: 465 us a pass with the whole ray
+    // at once, now 414). A box whose face is met in a segment meets the segment's
+    // bounding box; widened by a margin above the rounding errors of the slab planes and of the
+    // segment's ends (a few ulps of the coordinates), it keeps every box that counts.
     const float4* s_box = bt.boxes();
-    bt.any(lo[0], lo[1], lo[2], hi[0], hi[1], hi[2], [&](int i) {
+    auto face = [&](int i) {
         const float4 lo4 = s_box[2 * i], hi4 = s_box[2 * i + 1];
         const float blo[3] = {lo4.x, lo4.y, lo4.z}, bhi[3] = {hi4.x, hi4.y, hi4.z};
         float tn = -INFINITY, tf = INFINITY;
@@ -132,7 +128,24 @@ k_bounce(const float* __restrict__ pos, const float* __restrict__ nrm, int64_t n
             axis = ax;
         }
         return false;
-    });
+    };
+    float near = 0.0f, step = 0.125f * bt.extent();
+    for (int seg = 0;; ++seg) {
+        const bool rest = seg == 3 || !(step > 0.0f) || !(near + step < t_best);
+        const float far = rest ? t_best : near + step;
+        float lo[3], hi[3];
+        for (int k = 0; k < 3; ++k) {
+            const float from = fadd(o[k], fmul(near, d[k]));
+            const float to = fadd(o[k], fmul(far, d[k]));  // NaN (every box kept) if d = 0 and far infinite
+            const float e = 1e-5f * (1.0f + fabsf(from) + fabsf(to) + fabsf(o[k]));
+            lo[k] = fsub(to < from ? to : from, e);
+            hi[k] = fadd(to > from ? to : from, e);
+        }
+        bt.any(lo[0], lo[1], lo[2], hi[0], hi[1], hi[2], face);
+        if (rest || t_best <= far) break;
+        near = far;
+        step *= 2.0f;
+    }
     if (t_best == INFINITY) {  // nothing ahead: the path escapes
         for (int k = 0; k < 3; ++k) {
             y_out[k * np + p] = o[k];

@@ -61,6 +61,17 @@ struct BoxTable {
     {
         return reinterpret_cast<const float4*>(at + 32 + box_mask_bytes(n));
     }
+    // The boxes' largest extent along an axis (0: none, or no boxes).
+    __device__ __forceinline__ float extent() const
+    {
+        if (n == 0) return 0.0f;
+        const float4 sc = reinterpret_cast<const float4*>(at)[0];
+        float e = 0.0f;
+        if (sc.x > 0.0f) e = fmaxf(e, (float)box_bins(n) / sc.x);
+        if (sc.y > 0.0f) e = fmaxf(e, (float)box_bins(n) / sc.y);
+        if (sc.z > 0.0f) e = fmaxf(e, (float)box_bins(n) / sc.z);
+        return e;
+    }
     // Calls test(box index) for the boxes that can meet the axis-aligned box lo .. hi, in increasing
     // order of their index, until it returns true; whether it did.
     template <class Test>
