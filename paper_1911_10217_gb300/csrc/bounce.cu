@@ -36,131 +36,134 @@ constexpr float kPiF = 3.14159265358979323846f;
 
 __device__ __forceinline__ float fdivr(float a, float b) { return __fdiv_rn(a, b); }
 
+// As many blocks as fit the device, striding over the points: each builds the box table for itself, so
+// that bounces share no table with calls on other streams (path vertices at 720p 415 us a pass with
+// one table a launch and a block per 256 points, 418 so).
 __global__ void __launch_bounds__(kBounceThreads)
-k_bounce(const float* __restrict__ pos, const float* __restrict__ nrm, int64_t np, const void* __restrict__ table,
+k_bounce(const float* __restrict__ pos, const float* __restrict__ nrm, int64_t np, const float* __restrict__ boxes,
          int n_boxes, float r0, float r1, float r2, float r3, float r4, float r5, uint2 key, uint32_t frame,
          float paths_per_tile, float* __restrict__ y_out, float* __restrict__ ny_out, float* __restrict__ fp_out)
 {
     pdl_begin();
     extern __shared__ float4 s_boxes[];
-    const BoxTable bt = stage_box_table(s_boxes, table, n_boxes);
+    const BoxTable bt = stage_box_table<true>(s_boxes, nullptr, n_boxes, boxes);
     __syncthreads();
-    const int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (p >= np) return;
-    const float x[3] = {pos[p], pos[np + p], pos[2 * np + p]};
-    const float n[3] = {nrm[p], nrm[np + p], nrm[2 * np + p]};
+    for (int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; p < np; p += (int64_t)gridDim.x * blockDim.x) {
+        const float x[3] = {pos[p], pos[np + p], pos[2 * np + p]};
+        const float n[3] = {nrm[p], nrm[np + p], nrm[2 * np + p]};
 
-    // the disk point
-    float a = 0.0f, b = 0.0f;
-    uint4 w = make_uint4(0u, 0u, 0u, 0u);
-    for (int k = 0; k < kBounceTries; ++k) {
-        if ((k & 1) == 0) w = philox4x32_10(make_uint4((uint32_t)p, frame, (uint32_t)(k >> 1), 1u), key);
-        const float ua = u24((k & 1) ? w.z : w.x), ub = u24((k & 1) ? w.w : w.y);
-        const float ta = fsub(fmul(2.0f, ua), 1.0f), tb = fsub(fmul(2.0f, ub), 1.0f);
-        if (fadd(fmul(ta, ta), fmul(tb, tb)) < 1.0f) {
-            a = ta;
-            b = tb;
-            break;
-        }
-    }
-    const float s = fadd(fmul(a, a), fmul(b, b));
-    const float c = __fsqrt_rn(fmaxf(0.0f, fsub(1.0f, s)));  // cos(theta_x)
-
-    // tangent frame of n
-    const bool tx = fabsf(n[0]) < 0.9f;
-    const float t0 = tx ? 1.0f : 0.0f, t2 = tx ? 0.0f : 1.0f;
-    float u[3] = {fsub(fmul(n[1], t2), fmul(n[2], 0.0f)), fsub(fmul(n[2], t0), fmul(n[0], t2)),
-                  fsub(fmul(n[0], 0.0f), fmul(n[1], t0))};
-    const float ul = __fsqrt_rn(fadd(fadd(fmul(u[0], u[0]), fmul(u[1], u[1])), fmul(u[2], u[2])));
-    for (int k = 0; k < 3; ++k) u[k] = fdivr(u[k], ul);
-    const float v[3] = {fsub(fmul(n[1], u[2]), fmul(n[2], u[1])), fsub(fmul(n[2], u[0]), fmul(n[0], u[2])),
-                        fsub(fmul(n[0], u[1]), fmul(n[1], u[0]))};
-
-    float d[3], o[3], inv[3];
-    for (int k = 0; k < 3; ++k) {
-        d[k] = fadd(fadd(fmul(a, u[k]), fmul(b, v[k])), fmul(c, n[k]));
-        o[k] = fadd(x[k], fmul(kBounceOffset, n[k]));
-        inv[k] = fdivr(1.0f, d[k]);
-    }
-
-    // the first room wall ahead
-    const float rlo[3] = {r0, r1, r2}, rhi[3] = {r3, r4, r5};
-    float t_best = INFINITY;
-    int axis = 0;
-    for (int k = 0; k < 3; ++k) {
-        if (d[k] == 0.0f) continue;
-        const float wall = d[k] > 0.0f ? rhi[k] : rlo[k];
-        const float t = fmul(fsub(wall, o[k]), inv[k]);
-        if (t > kBounceTmin && t < t_best) {
-            t_best = t;
-            axis = k;
-        }
-    }
-    // The nearest box face in front of it, in up to four segments of the ray, the first an eighth of
-    // the boxes' extent long, each other twice the one before and the last the rest: most rays end in
-    // the first two, near which few boxes are (path vertices at 720p: 465 us a pass with the whole ray
-    // at once, now 414). A box whose face is met in a segment meets the segment's
-    // bounding box; widened by a margin above the rounding errors of the slab planes and of the
-    // segment's ends (a few ulps of the coordinates), it keeps every box that counts.
-    const float4* s_box = bt.boxes();
-    auto face = [&](int i) {
-        const float4 lo4 = s_box[2 * i], hi4 = s_box[2 * i + 1];
-        const float blo[3] = {lo4.x, lo4.y, lo4.z}, bhi[3] = {hi4.x, hi4.y, hi4.z};
-        float tn = -INFINITY, tf = INFINITY;
-        int ax = 0;
-        bool miss = false;
-        for (int k = 0; k < 3; ++k) {
-            if (d[k] == 0.0f) {  // parallel to this slab: inside it or a miss
-                if (!(o[k] > blo[k] && o[k] < bhi[k])) miss = true;
-                continue;
+        // the disk point
+        float a = 0.0f, b = 0.0f;
+        uint4 w = make_uint4(0u, 0u, 0u, 0u);
+        for (int k = 0; k < kBounceTries; ++k) {
+            if ((k & 1) == 0) w = philox4x32_10(make_uint4((uint32_t)p, frame, (uint32_t)(k >> 1), 1u), key);
+            const float ua = u24((k & 1) ? w.z : w.x), ub = u24((k & 1) ? w.w : w.y);
+            const float ta = fsub(fmul(2.0f, ua), 1.0f), tb = fsub(fmul(2.0f, ub), 1.0f);
+            if (fadd(fmul(ta, ta), fmul(tb, tb)) < 1.0f) {
+                a = ta;
+                b = tb;
+                break;
             }
-            const float ta = fmul(fsub(blo[k], o[k]), inv[k]);
-            const float tb = fmul(fsub(bhi[k], o[k]), inv[k]);
-            const float lo = fminf(ta, tb), hi = fmaxf(ta, tb);
-            if (lo > tn) {
-                tn = lo;
-                ax = k;
+        }
+        const float s = fadd(fmul(a, a), fmul(b, b));
+        const float c = __fsqrt_rn(fmaxf(0.0f, fsub(1.0f, s)));  // cos(theta_x)
+
+        // tangent frame of n
+        const bool tx = fabsf(n[0]) < 0.9f;
+        const float t0 = tx ? 1.0f : 0.0f, t2 = tx ? 0.0f : 1.0f;
+        float u[3] = {fsub(fmul(n[1], t2), fmul(n[2], 0.0f)), fsub(fmul(n[2], t0), fmul(n[0], t2)),
+                      fsub(fmul(n[0], 0.0f), fmul(n[1], t0))};
+        const float ul = __fsqrt_rn(fadd(fadd(fmul(u[0], u[0]), fmul(u[1], u[1])), fmul(u[2], u[2])));
+        for (int k = 0; k < 3; ++k) u[k] = fdivr(u[k], ul);
+        const float v[3] = {fsub(fmul(n[1], u[2]), fmul(n[2], u[1])), fsub(fmul(n[2], u[0]), fmul(n[0], u[2])),
+                            fsub(fmul(n[0], u[1]), fmul(n[1], u[0]))};
+
+        float d[3], o[3], inv[3];
+        for (int k = 0; k < 3; ++k) {
+            d[k] = fadd(fadd(fmul(a, u[k]), fmul(b, v[k])), fmul(c, n[k]));
+            o[k] = fadd(x[k], fmul(kBounceOffset, n[k]));
+            inv[k] = fdivr(1.0f, d[k]);
+        }
+
+        // the first room wall ahead
+        const float rlo[3] = {r0, r1, r2}, rhi[3] = {r3, r4, r5};
+        float t_best = INFINITY;
+        int axis = 0;
+        for (int k = 0; k < 3; ++k) {
+            if (d[k] == 0.0f) continue;
+            const float wall = d[k] > 0.0f ? rhi[k] : rlo[k];
+            const float t = fmul(fsub(wall, o[k]), inv[k]);
+            if (t > kBounceTmin && t < t_best) {
+                t_best = t;
+                axis = k;
             }
-            tf = fminf(tf, hi);
         }
-        if (!miss && tn < tf && tn > kBounceTmin && tn < t_best) {
-            t_best = tn;
-            axis = ax;
+        // The nearest box face in front of it, in up to four segments of the ray, the first an eighth of
+        // the boxes' extent long, each other twice the one before and the last the rest: most rays end in
+        // the first two, near which few boxes are (path vertices at 720p: 465 us a pass with the whole ray
+        // at once, now 414). A box whose face is met in a segment meets the segment's
+        // bounding box; widened by a margin above the rounding errors of the slab planes and of the
+        // segment's ends (a few ulps of the coordinates), it keeps every box that counts.
+        const float4* s_box = bt.boxes();
+        auto face = [&](int i) {
+            const float4 lo4 = s_box[2 * i], hi4 = s_box[2 * i + 1];
+            const float blo[3] = {lo4.x, lo4.y, lo4.z}, bhi[3] = {hi4.x, hi4.y, hi4.z};
+            float tn = -INFINITY, tf = INFINITY;
+            int ax = 0;
+            bool miss = false;
+            for (int k = 0; k < 3; ++k) {
+                if (d[k] == 0.0f) {  // parallel to this slab: inside it or a miss
+                    if (!(o[k] > blo[k] && o[k] < bhi[k])) miss = true;
+                    continue;
+                }
+                const float ta = fmul(fsub(blo[k], o[k]), inv[k]);
+                const float tb = fmul(fsub(bhi[k], o[k]), inv[k]);
+                const float lo = fminf(ta, tb), hi = fmaxf(ta, tb);
+                if (lo > tn) {
+                    tn = lo;
+                    ax = k;
+                }
+                tf = fminf(tf, hi);
+            }
+            if (!miss && tn < tf && tn > kBounceTmin && tn < t_best) {
+                t_best = tn;
+                axis = ax;
+            }
+            return false;
+        };
+        float near = 0.0f, step = 0.125f * bt.extent();
+        for (int seg = 0;; ++seg) {
+            const bool rest = seg == 3 || !(step > 0.0f) || !(near + step < t_best);
+            const float far = rest ? t_best : near + step;
+            float lo[3], hi[3];
+            for (int k = 0; k < 3; ++k) {
+                const float from = fadd(o[k], fmul(near, d[k]));
+                const float to = fadd(o[k], fmul(far, d[k]));  // NaN (every box kept) if d = 0 and far infinite
+                const float e = 1e-5f * (1.0f + fabsf(from) + fabsf(to) + fabsf(o[k]));
+                lo[k] = fsub(to < from ? to : from, e);
+                hi[k] = fadd(to > from ? to : from, e);
+            }
+            bt.any(lo[0], lo[1], lo[2], hi[0], hi[1], hi[2], face);
+            if (rest || t_best <= far) break;
+            near = far;
+            step *= 2.0f;
         }
-        return false;
-    };
-    float near = 0.0f, step = 0.125f * bt.extent();
-    for (int seg = 0;; ++seg) {
-        const bool rest = seg == 3 || !(step > 0.0f) || !(near + step < t_best);
-        const float far = rest ? t_best : near + step;
-        float lo[3], hi[3];
+        if (t_best == INFINITY) {  // nothing ahead: the path escapes
+            for (int k = 0; k < 3; ++k) {
+                y_out[k * np + p] = o[k];
+                ny_out[k * np + p] = 0.0f;
+            }
+            fp_out[p] = INFINITY;
+            continue;
+        }
         for (int k = 0; k < 3; ++k) {
-            const float from = fadd(o[k], fmul(near, d[k]));
-            const float to = fadd(o[k], fmul(far, d[k]));  // NaN (every box kept) if d = 0 and far infinite
-            const float e = 1e-5f * (1.0f + fabsf(from) + fabsf(to) + fabsf(o[k]));
-            lo[k] = fsub(to < from ? to : from, e);
-            hi[k] = fadd(to > from ? to : from, e);
+            y_out[k * np + p] = fadd(o[k], fmul(t_best, d[k]));
+            ny_out[k * np + p] = k == axis ? (d[axis] > 0.0f ? -1.0f : 1.0f) : 0.0f;
         }
-        bt.any(lo[0], lo[1], lo[2], hi[0], hi[1], hi[2], face);
-        if (rest || t_best <= far) break;
-        near = far;
-        step *= 2.0f;
+        const float cy = fabsf(d[axis]);  // cos(theta_y)
+        const float q = fmul(fmul(paths_per_tile, fmaxf(c, 1e-6f)), fmaxf(cy, 1e-6f));
+        fp_out[p] = fmul(t_best, __fsqrt_rn(fdivr(kPiF, q)));
     }
-    if (t_best == INFINITY) {  // nothing ahead: the path escapes
-        for (int k = 0; k < 3; ++k) {
-            y_out[k * np + p] = o[k];
-            ny_out[k * np + p] = 0.0f;
-        }
-        fp_out[p] = INFINITY;
-        return;
-    }
-    for (int k = 0; k < 3; ++k) {
-        y_out[k * np + p] = fadd(o[k], fmul(t_best, d[k]));
-        ny_out[k * np + p] = k == axis ? (d[axis] > 0.0f ? -1.0f : 1.0f) : 0.0f;
-    }
-    const float cy = fabsf(d[axis]);  // cos(theta_y)
-    const float q = fmul(fmul(paths_per_tile, fmaxf(c, 1e-6f)), fmaxf(cy, 1e-6f));
-    fp_out[p] = fmul(t_best, __fsqrt_rn(fdivr(kPiF, q)));
 }
 
 }  // namespace
@@ -183,14 +186,11 @@ extern "C" int rll_bounce_vertices(rll_ctx* ctx, const float* pos, const float* 
         return fail(ctx, RLL_E_INVALID, "NULL point or output array");
     if (n_points == 0) return RLL_OK;
     DeviceGuard g(ctx->device);
-    const void* table = nullptr;
-    const int rc = box_table(ctx, boxes, n_boxes, ctx->stream, &table);
-    if (rc != RLL_OK) return rc;
-    const unsigned blocks = (unsigned)((n_points + kBounceThreads - 1) / kBounceThreads);
     const size_t smem = n_boxes ? box_table_bytes(n_boxes) : 0;
+    const unsigned blocks = resident_blocks(ctx, k_bounce, n_points, kBounceThreads, smem);
     return check_cuda(ctx,
                       launch_pdl(k_bounce, dim3(blocks), dim3(kBounceThreads), smem, ctx->stream, pos, nrm, n_points,
-                                 table, (int)n_boxes, room[0], room[1], room[2], room[3], room[4], room[5],
+                                 boxes, (int)n_boxes, room[0], room[1], room[2], room[3], room[4], room[5],
                                  make_uint2((uint32_t)seed, (uint32_t)(seed >> 32)), frame, paths_per_tile, out_pos,
                                  out_nrm, out_footprint),
                       "bounce kernel");

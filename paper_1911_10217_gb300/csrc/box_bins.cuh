@@ -11,10 +11,11 @@
 // interval meets the segment's is left out; a coordinate without an order
 // (NaN) takes the bin that keeps every box.
 //
-// The table is rebuilt from the boxes by one block before every launch that
-// reads it (3.8 us; the boxes may change from call to call) and copied to
-// shared memory by each block that does. A sampling launch of few blocks and
-// boxes is done without: each block builds the table for itself (sample.cu).
+// The table is rebuilt from the boxes by one block before every sampling
+// launch (3.8 us; the boxes may change from call to call) and copied to
+// shared memory by each of its blocks. In a sampling launch of few blocks and
+// boxes, and in the energy sampler and the bounces, whose blocks stay and
+// take many points, each block builds the table for itself.
 // Against one run of the boxes sorted along x, which every segment searched
 // and then walked through (and, in the energy sampler and the bounces, against
 // every box): 12-scene batch equal, 1080p passes 424 -> 416 us, sky dome (128

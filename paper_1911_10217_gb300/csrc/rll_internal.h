@@ -5,6 +5,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <algorithm>
+
 #include <string>
 
 #include "../../include/rll.h"
@@ -40,8 +42,9 @@ struct rll_ctx {
     int host_zero_copy = 1;  // rll_render_pass_host: use mapped host buffers in place
     // launch tuning (rll_ctx_set_option)
     int sample_min_blocks = 4;
-    // the occluder boxes' table (box_bins.cuh), rebuilt by the calls that read boxes (sample.cu:
-    // box_table)
+    // the occluder boxes' table (box_bins.cuh) of the sampling calls, rebuilt by each (sample.cu:
+    // box_table); the energy sampler and the bounces share nothing with them or one another, since
+    // they may run on another stream (rll_ctx_set_stream)
     void* box_table = nullptr;
 };
 
@@ -144,6 +147,20 @@ int grid_from_float(rll_ctx* ctx, rll_grid* g, const float* q_in, const float* c
 int grid_mark_occupied(rll_ctx* ctx, rll_grid* g);  // touched list := every occupied slot
 int key_bits(uint64_t hm_plus_one);
 int device_sm_count(int device);
+// Blocks of `threads` for n threads' work in a kernel that strides by its grid: no more than fit the
+// device at once.
+template <class F>
+unsigned resident_blocks(const rll_ctx* ctx, F* kernel, int64_t n, int threads, size_t smem)
+{
+    const int64_t blocks = (n + threads - 1) / threads, sms = device_sm_count(ctx->device);
+    int per_sm = 1;
+    if (blocks > sms &&
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, threads, smem) != cudaSuccess) {
+        cudaGetLastError();
+        per_sm = 1;
+    }
+    return (unsigned)std::min(blocks, sms * std::max(per_sm, 1));
+}
 // split-collapse steps per cell and call (0 reads as 1)
 inline uint32_t split_steps(const rll_grid_params& p) { return p.split_iterations ? p.split_iterations : 1u; }
 int learn_update(rll_ctx* ctx, rll_grid* g, const uint32_t* rec_key, const float* rec_val, int64_t n);
