@@ -37,9 +37,9 @@ UNIT = "light samples/s"
 PEAKS_FALLBACK = {"hbm_gbs": 6800.0, "bf16_tflops": 1900.0}
 SM_COUNT = 152
 # DRAM bytes (read + write) of one k_sample launch on this workload, from one ncu capture of it
-# (76.30 MB read + 20.90 MB written; kernel as of commit e94a3a1); None whenever the sampling
+# (76.23 MB read + 15.93 MB written; kernel as of commit c41eaaf); None whenever the sampling
 # kernel has changed since that capture
-K_SAMPLE_DRAM_BYTES = 97.19e6
+K_SAMPLE_DRAM_BYTES = 92.16e6
 FP32_LANES_PER_SM = 128
 
 
