@@ -285,7 +285,7 @@ template <int P, int MODE, int MINB>
 cudaError_t launch_sample_t(rll_batch* b, cudaStream_t s)
 {
     int per_sm = 0;
-    const size_t smem = box_table_bytes(std::max(b->max_boxes, 1));
+    const size_t smem = box_table_room(std::max(b->max_boxes, 1));  // the items' counts differ
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_sample_batched<P, MODE, MINB>, kBatchThreads, smem);
     const int blocks = std::max(1, per_sm) * device_sm_count(b->device);
     cudaError_t e = cudaMemsetAsync(b->d_work, 0, sizeof(uint32_t), s);

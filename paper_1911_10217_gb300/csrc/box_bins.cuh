@@ -42,6 +42,23 @@ __host__ __device__ constexpr size_t box_table_bytes(int n) { return 32u + box_m
 constexpr size_t kMaxBoxTable = box_table_bytes(kMaxBoxes);
 static_assert(box_table_bytes(256) < kMaxBoxTable && kMaxBoxTable % 16 == 0, "box table size");
 
+// Bytes that hold the table of any number of boxes up to n, which box_table_bytes(n) does not: the
+// bins halve above 256 boxes, where 257 take 12 096 bytes and 256 take 14 368.
+__host__ __device__ constexpr size_t box_table_room(int n)
+{
+    return n > 256 && box_table_bytes(n) < box_table_bytes(256) ? box_table_bytes(256) : box_table_bytes(n);
+}
+constexpr bool box_table_room_holds()
+{
+    size_t most = 0;
+    for (int n = 0; n <= kMaxBoxes; ++n) {
+        most = box_table_bytes(n) > most ? box_table_bytes(n) : most;
+        if (box_table_room(n) < most) return false;
+    }
+    return box_table_room(kMaxBoxes) == kMaxBoxTable;
+}
+static_assert(box_table_room_holds(), "a smaller table exceeds the room of a larger one");
+
 // Bin of a coordinate whose scaled value is t: as a lower end (NaN: the first bin) or an upper end
 // (NaN: the last).
 __device__ __forceinline__ int box_bin_lo(float t, int bins)
