@@ -458,8 +458,9 @@ __device__ __forceinline__ void sample_point(const SampleArgs& a, int64_t p, con
 }
 
 // Floats of shared memory that a warp of sample_points needs: a round's estimates, and the sums of
-// the point that the round ends in.
-constexpr int kWarpEst = 3 * 32 + 3;
+// the point that a round ends in, in one place for even rounds and one for odd ones (a round reads
+// the one before's while other lanes write its own).
+constexpr int kWarpEst = 3 * 32 + 2 * 3;
 
 // How a launch of n_points points of spp samples on a device that holds `warps` warps splits them:
 // the points a warp of sample_points takes at a time, or 0 for a thread a point. The cost of a split
@@ -511,13 +512,14 @@ __device__ __forceinline__ void sample_points(const SampleArgs& a, int64_t p0, u
         for (int k = 0; k < 3; ++k) s_est[32 * k + lane] = est[k];
         __syncwarp();
         const uint32_t end = min(base + 32, total), q0 = base / spp, q1 = (end - 1) / spp;
+        const uint32_t carry = 96 + 3 * ((base >> 5) & 1u), before = 96 + 99 - carry;
         for (uint32_t t = lane; t < 3 * (q1 - q0 + 1); t += 32) {
             const uint32_t q = q0 + t / 3, ch = t % 3;
             const uint32_t from = max(q * spp, base), to = min((q + 1) * spp, end);
-            float acc = from == q * spp ? 0.0f : s_est[96 + ch];
+            float acc = from == q * spp ? 0.0f : s_est[before + ch];
             for (uint32_t j = from; j < to; ++j) acc += s_est[32 * ch + (j - base)];
             if (to == (q + 1) * spp) a.rgb[ch * np + p0 + q] = acc * inv_spp;
-            else s_est[96 + ch] = acc;
+            else s_est[carry + ch] = acc;
         }
         __syncwarp();
     }
