@@ -189,7 +189,7 @@ struct rll_batch {
     uint32_t* touched_start = nullptr; // [cap_cells]
     uint32_t* touched_len = nullptr;   // [cap_cells]
     uint32_t* lists = nullptr;         // [2 cap_cells] cells for the block paths
-    uint32_t* n_touched = nullptr;     // [8] learning counters
+    uint32_t* n_touched = nullptr;     // [kLearnCounters] learning counters
     int max_boxes = 0;
     uint32_t* status = nullptr;
     char* box_tables = nullptr;        // [cap_items][kMaxBoxTable] the tables of the items' boxes
@@ -321,7 +321,7 @@ cudaError_t launch_sample(rll_batch* b, cudaStream_t s)
 template <int P>
 cudaError_t launch_learn_t(rll_batch* b, cudaStream_t s, bool do_split)
 {
-    if (b->n_records == 0) return cudaMemsetAsync(b->n_touched, 0, 8 * sizeof(uint32_t), s);
+    if (b->n_records == 0) return cudaMemsetAsync(b->n_touched, 0, kLearnCounters * sizeof(uint32_t), s);
     const int sms = device_sm_count(b->device);
     const BatchDec dec{b->total_cells << kBatchClusterBits};
     const BatchRows<P> rows{b->d_items, b->n, b->d_cell_prefix};
@@ -378,7 +378,7 @@ int rll_batch_reserve(rll_ctx* ctx, int32_t max_items, int64_t max_records, int6
     if (e == cudaSuccess) e = cudaMalloc((void**)&b->touched_start, 4 * (size_t)max_cells);
     if (e == cudaSuccess) e = cudaMalloc((void**)&b->touched_len, 4 * (size_t)max_cells);
     if (e == cudaSuccess) e = cudaMalloc((void**)&b->lists, 8 * (size_t)max_cells);
-    if (e == cudaSuccess) e = cudaMalloc((void**)&b->n_touched, 8 * sizeof(uint32_t));
+    if (e == cudaSuccess) e = cudaMalloc((void**)&b->n_touched, kLearnCounters * sizeof(uint32_t));
     if (e == cudaSuccess) e = cudaMalloc((void**)&b->box_tables, kMaxBoxTable * (size_t)max_items);
     if (e == cudaSuccess) e = cudaMemsetAsync(b->cursor, 0, 4 * (size_t)max_cells, ctx->stream);
     // the learning step's shared-memory opt-in, now rather than during a graph capture
@@ -392,7 +392,7 @@ int rll_batch_reserve(rll_ctx* ctx, int32_t max_items, int64_t max_records, int6
     if (e == cudaSuccess) e = cudaMalloc((void**)&b->d_items, sizeof(BatchItemDev) * max_items);
     if (e == cudaSuccess) e = cudaMalloc((void**)&b->d_tile_prefix, 4 * (max_items + 1));
     if (e == cudaSuccess) e = cudaMalloc((void**)&b->d_cell_prefix, 4 * (max_items + 1));
-    if (e == cudaSuccess) e = cudaMemsetAsync(b->n_touched, 0, 8 * sizeof(uint32_t), ctx->stream);
+    if (e == cudaSuccess) e = cudaMemsetAsync(b->n_touched, 0, kLearnCounters * sizeof(uint32_t), ctx->stream);
     if (e == cudaSuccess) {
         const size_t items_b = (sizeof(BatchItemDev) * max_items + 255) & ~(size_t)255;
         const size_t pre_b = (4 * ((size_t)max_items + 1) + 255) & ~(size_t)255;

@@ -11,6 +11,7 @@
 
 #include "learn_core.cuh"
 #include "rll_device.cuh"
+#include "rll_internal.h"
 
 namespace rll {
 namespace {  // every translation unit that includes this header gets its own copies
@@ -25,11 +26,13 @@ struct RowRef {
 };
 
 // ---------------------------------------------------------------- bucketed learning
-// counters ctr[8]: [0] touched cells, [1] bucket space claimed, [2] cells for
+// counters ctr[kLearnCounters]: [0] touched cells, [1] bucket space claimed, [2] cells for
 // the sorting block path, [3] cells for the two-warp path, [4] [5] [7] work
 // counters of the block, warp and two-warp phases, [6] cells for the grouping
-// block path; lists[2 * cells]: the grouping list (two-warp cells from the
+// block path, [8] [9] flags: claim complete, scatter complete (kClaimed,
+// kScattered: see k_learn_buckets); lists[2 * cells]: the grouping list (two-warp cells from the
 // front, block cells from the back), then the sorting list
+constexpr int kClaimed = 8, kScattered = 9;
 constexpr int kBucketThreads = 256;
 constexpr int kTilesPerWarp = 4;         // 32-record tiles one warp counts / scatters
 constexpr uint32_t kWarpBucket = 240;    // records of a cell one warp orders in shared memory
@@ -198,9 +201,14 @@ struct Bucket {
 template <class Dec>
 __global__ void __launch_bounds__(kBucketThreads)
 k_bucket_scatter(const uint32_t* __restrict__ rec_key, const float* __restrict__ rec_val, int64_t n, Dec dec,
-                 const uint32_t* __restrict__ cursor, const uint32_t* __restrict__ rank, Bucket bucket)
+                 const uint32_t* __restrict__ cursor, const uint32_t* __restrict__ rank, Bucket bucket,
+                 uint32_t* __restrict__ ctr)
 {
-    pdl_begin();
+    pdl_wait();
+    if (threadIdx.x == 0) {  // the flag before the block's release: see k_learn_buckets
+        if (blockIdx.x == 0) store_release(ctr + kClaimed, 1u);
+        pdl_release();
+    }
     const int64_t i0 = (int64_t)blockIdx.x * kBucketThreads * kTilesPerWarp + threadIdx.x;
     uint32_t key[kTilesPerWarp], val[kTilesPerWarp], rk[kTilesPerWarp], at[kTilesPerWarp];
 #pragma unroll
@@ -240,7 +248,7 @@ k_bucket_small(const uint32_t* __restrict__ rec_key, const float* __restrict__ r
 {
     pdl_wait();
     const uint32_t lane = threadIdx.x & 31u, g = blockIdx.x * kSmallThreads + threadIdx.x;
-    if (g < 8) ctr[g] = 0u;
+    if (g < (uint32_t)kLearnCounters) ctr[g] = 0u;
     __threadfence();
     cluster_sync();
     uint32_t key[kSmallItems], rank[kSmallItems];
@@ -282,7 +290,10 @@ k_bucket_small(const uint32_t* __restrict__ rec_key, const float* __restrict__ r
                 group_list, sort_list, cells);
     __threadfence();
     cluster_sync();
-    pdl_release();  // the next kernel reads the counts as soon as it starts
+    if (threadIdx.x == 0) {  // the flag before the block's release: see k_learn_buckets
+        if (blockIdx.x == 0) store_release(ctr + kClaimed, 1u);
+        pdl_release();
+    }
 #pragma unroll
     for (int u = 0; u < kSmallItems; ++u) {
         const uint32_t i = (uint32_t)u * (kSmallBlocks * kSmallThreads) + g;
@@ -588,19 +599,23 @@ struct LearnSmem {
 
 template <int P, int WARPS, int MINB, uint32_t CLUS, class Rows, class Split>
 __global__ void __launch_bounds__(WARPS * 32, MINB)
-k_learn_buckets(const Bucket bucket, uint32_t* __restrict__ ctr, const uint32_t* __restrict__ group_list,
-                const uint32_t* __restrict__ touched, const uint32_t* __restrict__ start,
-                const uint32_t* __restrict__ len, uint32_t* __restrict__ cursor, Rows rows, Split sp,
+k_learn_buckets(const Bucket bucket, uint32_t* ctr, const uint32_t* group_list, const uint32_t* touched,
+                const uint32_t* start, const uint32_t* len, uint32_t* __restrict__ cursor, Rows rows, Split sp,
                 uint32_t* __restrict__ status, uint32_t cells)
 {
     // Launched after k_learn_big, whose cells are others. Where it has cells, this kernel runs beside
-    // it: it starts when every block of k_learn_big has released it, that is when the scatter is
-    // complete and visible (each block waits for it first), and ends only when k_learn_big has, so
-    // that whatever follows this kernel follows both. Where it has none, k_learn_big releases this
-    // kernel at once and ends with the scatter, for which this kernel's blocks wait in their places.
-    // (The claim, which writes the counts, is complete before any block of the scatter, or of
-    // k_bucket_small, releases.)
-    const bool beside = *(volatile const uint32_t*)(ctr + 2) != 0u;
+    // it: it starts when every block of k_learn_big has released it, each after its wait for the
+    // scatter, and ends only when k_learn_big has, so that whatever follows this kernel follows both.
+    // Where it has none, k_learn_big releases this kernel at once and ends with the scatter, for which
+    // this kernel's blocks wait in their places.
+    // A release lets the next kernel start and makes nothing visible to it; that is done by two flags,
+    // cleared with the counters. kClaimed: block 0 of the scatter stores it behind its wait for the
+    // claim (k_bucket_small: behind the claim), before it releases; k_learn_big loads it and then reads
+    // its cells' count. kScattered: block 0 of k_learn_big, which has cells, stores it behind its wait
+    // for the scatter, before it releases; this kernel loads it, and so knows that it runs beside, and
+    // that counts, lists and buckets can be read (by ordinary loads: the lists' pointers are not
+    // restrict). A thread that does not see its flag waits for the kernel before its own.
+    const bool beside = load_acquire(ctr + kScattered) != 0u;
     if (!beside) pdl_wait();
     pdl_release();
     static_assert(WARPS == 6, "three warp pairs, named barriers 1 .. 3");
@@ -812,18 +827,21 @@ __device__ __forceinline__ void radix_pass(const unsigned long long* src, unsign
 template <int P, class Rows, class Split>
 __global__ void __launch_bounds__(kBigThreads)
 k_learn_big(const Bucket bucket, unsigned long long* __restrict__ wide, const float* __restrict__ rec_val,
-            const uint32_t* __restrict__ ctr,
-            const uint32_t* __restrict__ touched, const uint32_t* __restrict__ start,
-            const uint32_t* __restrict__ len, const uint32_t* __restrict__ big, uint32_t* __restrict__ cursor,
-            Rows rows, Split sp, uint32_t* __restrict__ status, uint32_t n_ids)
+            uint32_t* ctr, const uint32_t* touched, const uint32_t* start, const uint32_t* len, const uint32_t* big,
+            uint32_t* __restrict__ cursor, Rows rows, Split sp, uint32_t* __restrict__ status, uint32_t n_ids)
 {
-    const uint32_t n_big = *(volatile const uint32_t*)(ctr + 2);  // complete: see k_learn_buckets
+    if (load_acquire(ctr + kClaimed) == 0u) pdl_wait();  // see k_learn_buckets
+    const uint32_t n_big = *(volatile const uint32_t*)(ctr + 2);
     if (n_big == 0) {
         pdl_release();
         pdl_wait();
         return;
     }
-    pdl_begin();
+    pdl_wait();
+    if (threadIdx.x == 0) {
+        if (blockIdx.x == 0) store_release(ctr + kScattered, 1u);
+        pdl_release();
+    }
     extern __shared__ unsigned long long s_rec[];      // two tiles, then the warps' digit counters
     uint32_t* s_wc = reinterpret_cast<uint32_t*>(s_rec + 2 * kBlockSort);
     __shared__ float s_q[kMaxCut], s_c[kMaxCut];
@@ -921,12 +939,13 @@ inline size_t bucketed_scratch_bytes(int64_t n)
 }
 
 // Enqueues the whole learning step for n >= 1 records (cut sizes up to
-// max_cut), every kernel with the programmatic launch dependency (each waits
-// for its predecessor first). Clears ctr[0..7] first; the caller holds
+// max_cut), every kernel with the programmatic launch dependency (those up to
+// the scatter wait for their predecessors first, the last two as k_learn_buckets
+// says). Clears ctr first; the caller holds
 // `cursor` [cells] at zero (left at zero again); touched, start,
 // len [cells] and lists [2 * cells] are outputs and scratch. Counters: ctr[0]
 // touched cells, [1] claimed records, [2] sorting list, [3] two-warp list,
-// [6] block list, [4] [5] [7] work counters of k_learn_buckets.
+// [6] block list, [4] [5] [7] work counters of k_learn_buckets, [8] [9] flags.
 template <int P, class Dec, class Rows, class Split = NoSplit>
 cudaError_t launch_bucketed_learn(cudaStream_t s, int device, int sms, const uint32_t* rec_key,
                                   const float* rec_val, int64_t n, Dec dec, Rows rows, uint32_t cells,
@@ -952,7 +971,7 @@ cudaError_t launch_bucketed_learn(cudaStream_t s, int device, int sms, const uin
         e0 = launch_pdl(k_bucket_small<Dec>, dim3(kSmallBlocks), dim3(kSmallThreads), 0, s, rec_key, rec_val, (uint32_t)n,
                         dec, cursor, touched, ctr, start, len, group_list, sort_list, cells, bucket);
     } else {
-        e0 = cudaMemsetAsync(ctr, 0, 8 * sizeof(uint32_t), s);
+        e0 = cudaMemsetAsync(ctr, 0, kLearnCounters * sizeof(uint32_t), s);
         if (e0 == cudaSuccess)
             e0 = launch_pdl(k_bucket_count<Dec>, dim3(rblocks), dim3(kBucketThreads), 0, s, rec_key, n, dec, cursor,
                             touched, ctr, rank);
@@ -961,7 +980,7 @@ cudaError_t launch_bucketed_learn(cudaStream_t s, int device, int sms, const uin
                             len, group_list, sort_list, cells);
         if (e0 == cudaSuccess)
             e0 = launch_pdl(k_bucket_scatter<Dec>, dim3(rblocks), dim3(kBucketThreads), 0, s, rec_key, rec_val, n, dec,
-                            cursor, rank, bucket);
+                            cursor, rank, bucket, ctr);
     }
     if (e0 != cudaSuccess) return e0;
     // k_learn_big first, k_learn_buckets beside it: its blocks, few and long, take the place they need,

@@ -433,13 +433,27 @@ template <> struct Store<RLL_PREC_BF16> {
 // scheduled while the kernel before it on the stream is finishing; its first
 // statement is pdl_begin(): wait until that kernel (and so all earlier work)
 // has completed and its writes are visible, then let the next kernel be
-// scheduled in turn.
+// scheduled in turn. (Between the learning kernels some of this is said apart
+// and handed on by flags: see k_learn_buckets.)
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_release() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void pdl_begin()
 {
     pdl_wait();
     pdl_release();
+}
+
+// A flag between kernels that may run at once: what the thread that stores it has seen or written is
+// visible to the thread that loads the stored value.
+__device__ __forceinline__ void store_release(uint32_t* p, uint32_t v)
+{
+    asm volatile("st.release.gpu.global.u32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
+}
+__device__ __forceinline__ uint32_t load_acquire(const uint32_t* p)
+{
+    uint32_t v;
+    asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+    return v;
 }
 
 template <typename... KArgs, typename... Args>
