@@ -103,8 +103,13 @@ k_bounce(const float* __restrict__ pos, const float* __restrict__ nrm, int64_t n
         // the first two, near which few boxes are (path vertices at 720p: 465 us a pass with the whole ray
         // at once, now 414). A box whose face is met in a segment meets the segment's
         // bounding box; widened by a margin above the rounding errors of the slab planes and of the
-        // segment's ends (a few ulps of the coordinates), it keeps every box that counts.
+        // segment's ends (a few ulps of the coordinates), it keeps every box that counts. Of boxes met at
+        // the same distance the first counts, as if all were tested in turn: one that reaches back into
+        // an early segment and is met beyond it shortens the next ones, but is met again in the last,
+        // in its turn (its distance is raised by an ulp until then; told apart by their indices at every
+        // test instead, or left to the last segment altogether, 1080p bounces took 130 us, now 125).
         const float4* s_box = bt.boxes();
+        const float t_wall = t_best;
         auto face = [&](int i) {
             const float4 lo4 = s_box[2 * i], hi4 = s_box[2 * i + 1];
             const float blo[3] = {lo4.x, lo4.y, lo4.z}, bhi[3] = {hi4.x, hi4.y, hi4.z};
@@ -145,6 +150,7 @@ k_bounce(const float* __restrict__ pos, const float* __restrict__ nrm, int64_t n
             }
             bt.any(lo[0], lo[1], lo[2], hi[0], hi[1], hi[2], face);
             if (rest || t_best <= far) break;
+            if (t_best < t_wall) t_best = __uint_as_float(__float_as_uint(t_best) + 1u);
             near = far;
             step *= 2.0f;
         }

@@ -1,5 +1,5 @@
-"""Occluder sets whose table differs from the ordinary one: batches of items
-with different box counts (marked gpu)."""
+"""Occluder sets that the ordinary ones leave out: batches of items
+with different box counts, boxes met at the same distance (marked gpu)."""
 import dataclasses
 
 import numpy as np
@@ -44,3 +44,59 @@ def test_batch_of_mixed_box_counts(env, counts):
         # the tolerance of test_batch_matches_single_grid_path
         assert np.allclose(o["rgb"].cpu().numpy(), rgb.cpu().numpy(), rtol=1e-5, atol=1e-9)
     assert ctx.sync_status() == 0
+
+
+def bounce_ray(O, x, n, seed, point, frame):
+    """Origin, direction and reciprocal of a point's bounce in binary32, for a normal (0, 1, 0): the
+    tangent frame is (0, 0, -1), (-1, 0, 0)."""
+    f = np.float32
+    a = b = f(0)
+    for k in range(16):
+        w = O.philox4x32_10([point, frame, k >> 1, 1], [seed, 0])
+        ta, tb = (f(2) * (f(int(w[2 * (k & 1) + j]) >> 8) * f(2.0 ** -24)) - f(1) for j in (0, 1))
+        if f(ta * ta) + f(tb * tb) < f(1):
+            a, b = ta, tb
+            break
+    c = np.sqrt(f(1) - f(f(a * a) + f(b * b)))
+    d = np.array([-b, c, -a], f)
+    return np.asarray(x, f) + f(1e-4) * np.asarray(n, f), d, f(1) / d
+
+
+def test_bounce_on_two_boxes_at_the_same_distance(env):
+    """A ray that meets a side of one box and the underside of another at the same binary32 distance,
+    beyond the first segment: the box of the lower index counts, also where the other one reaches back
+    to the ray's origin and is tested first."""
+    O, rll, ctx, torch, dev = env["O"], env["rll"], env["ctx"], env["torch"], env["dev"]
+    f = np.float32
+    x, n, seed, frame, P = [0.51, 0.05, 0.5], [0.0, 1.0, 0.0], 9, 2, 4000
+    pos, nrm = (np.repeat(np.array(v, f)[:, None], P, 1) for v in (x, n))
+    corners = np.array([[0, 0, 0, .01, .01, .01], [.99, .99, .99, 1, 1, 1]], f)
+    t = lambda a: torch.from_numpy(np.ascontiguousarray(a)).to(dev)  # noqa: E731
+    tried = 0
+    for p in range(P):
+        o, d, inv = bounce_ray(O, x, n, seed, p, frame)
+        if not (0.01 < d[0] < 0.02 and abs(d[2]) < 0.5 and tried < 4):
+            continue
+        for y in np.linspace(0.6, 0.7, 400, dtype=f):
+            T = f(y - o[1]) * inv[1]
+            side = f(o[0] + T * d[0]) + np.arange(-40, 41).astype(f) * f(2.0 ** -24)
+            side = side[(side - o[0]).astype(f) * inv[0] == T]
+            if side.size:
+                break
+        else:
+            continue
+        tried += 1
+        z = float(o[2] + T * d[2])
+        above = np.array([o[0] - 0.02, y, z - 0.02, o[0] + 0.05, y + 0.1, z + 0.02], f)  # far from the origin
+        beside = np.array([side[0], 0.0, 0.0, side[0] + f(0.3), 1.0, 1.0], f)             # along the ray
+        axes = []
+        for boxes in ([above, beside, *corners], [*corners, beside, above]):
+            boxes = np.array(boxes, f)
+            want = [np.asarray(a, f) for a in O.bounce_vertices(pos, nrm, boxes, scenes.ROOM, seed, frame, 50.0)]
+            out = [torch.empty(3, P, device=dev), torch.empty(3, P, device=dev), torch.empty(P, device=dev)]
+            rll.bounce_vertices(ctx, t(pos), t(nrm), t(boxes), scenes.ROOM, seed, frame, 50.0, *out)
+            for got, w in zip(out, want):
+                assert np.array_equal(got.cpu().numpy(), w)
+            axes.append(int(np.argmax(np.abs(want[1][:, p]))))
+        assert axes == [1, 0]  # the two are at the same distance indeed
+    assert tried >= 2
