@@ -35,8 +35,9 @@ namespace {  // build_box_table is out of line: every translation unit has its o
 __host__ __device__ constexpr int box_bins(int n) { return n <= 256 ? 32 : 16; }
 __host__ __device__ constexpr int box_words(int n) { return (n + 63) / 64; }
 
-// Layout of the table: (scale xyz, 0) and (offset xyz, 0) as float4; masks [6][bins][words] of 64
-// bits, axis k's begin masks at 2k and its end masks at 2k + 1; boxes [n] as float4 (min), (max).
+// Layout of the table: (scale xyz, w) and (offset xyz, 0) as float4, w = 1 where a box has a minimum
+// above its maximum, else 0; masks [6][bins][words] of 64 bits, axis k's begin masks at 2k and its end
+// masks at 2k + 1; boxes [n] as float4 (min), (max).
 __host__ __device__ constexpr size_t box_mask_bytes(int n) { return 48u * (size_t)box_bins(n) * (size_t)box_words(n); }
 __host__ __device__ constexpr size_t box_table_bytes(int n) { return 32u + box_mask_bytes(n) + 32u * (size_t)n; }
 constexpr size_t kMaxBoxTable = box_table_bytes(kMaxBoxes);
@@ -79,6 +80,11 @@ struct BoxTable {
     {
         return reinterpret_cast<const float4*>(at + 32 + box_mask_bytes(n));
     }
+    // A box has a minimum above its maximum.
+    __device__ __forceinline__ bool swapped() const
+    {
+        return n > 0 && reinterpret_cast<const float4*>(at)[0].w != 0.0f;
+    }
     // The boxes' largest extent along an axis (0: none, or no boxes).
     __device__ __forceinline__ float extent() const
     {
@@ -117,6 +123,11 @@ struct BoxTable {
     }
 };
 
+// The ends of a box along axis k, lower and upper, also of one given the other way round (which the
+// slab tests take like any other).
+__device__ __forceinline__ float box_lower(const float* v, int k) { return v[3 + k] < v[k] ? v[3 + k] : v[k]; }
+__device__ __forceinline__ float box_upper(const float* v, int k) { return v[3 + k] < v[k] ? v[k] : v[3 + k]; }
+
 // Builds the table of n (1 .. kMaxBoxes) boxes [n][6] into out, by a whole block of at most 256
 // threads; s_mask: its masks in shared memory, or a scratch copy of them there (box_mask_bytes).
 __device__ __noinline__ void build_box_table(const float* __restrict__ boxes, int n, char* out, uint32_t* s_mask)
@@ -127,12 +138,14 @@ __device__ __noinline__ void build_box_table(const float* __restrict__ boxes, in
     for (int i = threadIdx.x; i < 6 * bins * words; i += blockDim.x) s_mask[i] = 0u;
     float lim[6] = {INFINITY, INFINITY, INFINITY, -INFINITY, -INFINITY, -INFINITY};
     float4* box = reinterpret_cast<float4*>(out + 32 + box_mask_bytes(n));
+    bool swapped = false;
     for (int b = threadIdx.x; b < n; b += blockDim.x) {
         const float* v = boxes + 6 * b;
         for (int k = 0; k < 3; ++k) {
-            lim[k] = fminf(lim[k], v[k]);
-            lim[3 + k] = fmaxf(lim[3 + k], v[3 + k]);
+            lim[k] = fminf(lim[k], box_lower(v, k));
+            lim[3 + k] = fmaxf(lim[3 + k], box_upper(v, k));
         }
+        swapped = swapped || v[3] < v[0] || v[4] < v[1] || v[5] < v[2];
         box[2 * b] = make_float4(v[0], v[1], v[2], 0.0f);
         box[2 * b + 1] = make_float4(v[3], v[4], v[5], 0.0f);
     }
@@ -145,7 +158,7 @@ __device__ __noinline__ void build_box_table(const float* __restrict__ boxes, in
         }
         if (lane == 0) s_lim[warp][k] = lim[k];
     }
-    __syncthreads();
+    swapped = __syncthreads_or(swapped);
     if (threadIdx.x < 3) {
         const int k = threadIdx.x;
         float lo = s_lim[0][k], hi = s_lim[0][3 + k];
@@ -161,13 +174,14 @@ __device__ __noinline__ void build_box_table(const float* __restrict__ boxes, in
     __syncthreads();
     if (threadIdx.x < 2) {
         const float* v = threadIdx.x ? s_off : s_scale;
-        reinterpret_cast<float4*>(out)[threadIdx.x] = make_float4(v[0], v[1], v[2], 0.0f);
+        const float w = threadIdx.x == 0 && swapped ? 1.0f : 0.0f;
+        reinterpret_cast<float4*>(out)[threadIdx.x] = make_float4(v[0], v[1], v[2], w);
     }
     for (int i = threadIdx.x; i < 3 * n; i += blockDim.x) {
         const int b = i / 3, k = i % 3;
         const float* v = boxes + 6 * b;
-        const int j0 = box_bin_lo(__fmaf_rn(v[k], s_scale[k], s_off[k]), bins);
-        const int j1 = box_bin_hi(__fmaf_rn(v[3 + k], s_scale[k], s_off[k]), bins);
+        const int j0 = box_bin_lo(__fmaf_rn(box_lower(v, k), s_scale[k], s_off[k]), bins);
+        const int j1 = box_bin_hi(__fmaf_rn(box_upper(v, k), s_scale[k], s_off[k]), bins);
         atomicOr(&s_mask[(2 * k * bins + j0) * words + (b >> 5)], 1u << (b & 31));
         atomicOr(&s_mask[((2 * k + 1) * bins + j1) * words + (b >> 5)], 1u << (b & 31));
     }

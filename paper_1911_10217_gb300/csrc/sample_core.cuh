@@ -120,6 +120,49 @@ __device__ __forceinline__ float seg_dir(float d)
     return fabsf(d) >= 0x1p-100f ? d : copysignf(0x1p-100f, d);
 }
 
+// Above the rounding error of the shadow test's slab planes (a few ulps of |o| + |y|).
+__device__ __forceinline__ float shadow_margin(float o, float y) { return 1e-5f * (1.0f + fabsf(o) + fabsf(y)); }
+
+// Whether the segment o + t d, t in (0, kShadowTmax), crosses a box (i = 1 / d, q = -o i).
+__device__ __forceinline__ bool slabs_cross(const float4& bmin, const float4& bmax, float i0, float i1, float i2,
+                                            float q0, float q1, float q2)
+{
+    const float ta0 = __fmaf_rn(bmin.x, i0, q0), tb0 = __fmaf_rn(bmax.x, i0, q0);
+    const float ta1 = __fmaf_rn(bmin.y, i1, q1), tb1 = __fmaf_rn(bmax.y, i1, q1);
+    const float ta2 = __fmaf_rn(bmin.z, i2, q2), tb2 = __fmaf_rn(bmax.z, i2, q2);
+    float tn = fmaxf(0.0f, fminf(ta0, tb0));
+    float tf = fminf(kShadowTmax, fmaxf(ta0, tb0));
+    tn = fmaxf(tn, fminf(ta1, tb1));
+    tf = fminf(tf, fmaxf(ta1, tb1));
+    tn = fmaxf(tn, fminf(ta2, tb2));
+    tf = fminf(tf, fmaxf(ta2, tb2));
+    return tn < tf;
+}
+
+namespace {
+// The shadow test of box sets in which a box has a minimum above its maximum: such a box counts only
+// where the segment's bounding box spans it (the ends compared as they are given). The table takes it
+// for the box between its ends, which is where it can meet a segment. Out of line and of no use to
+// other sets: 1080p sampling 320 us with and without it, energy sampler 87 (a mark at every box, tested
+// where a box blocks, cost the energy sampler 12 %; a call behind the test 2 to 5 % of the sampling).
+__device__ __noinline__ bool spanned_box_blocks(BoxTable bt, float o0, float o1, float o2, float y0, float y1,
+                                                float y2)
+{
+    const float i0 = fdiv(1.0f, seg_dir(fsub(y0, o0))), i1 = fdiv(1.0f, seg_dir(fsub(y1, o1))),
+                i2 = fdiv(1.0f, seg_dir(fsub(y2, o2)));
+    const float q0 = -fmul(o0, i0), q1 = -fmul(o1, i1), q2 = -fmul(o2, i2);
+    const float e0 = shadow_margin(o0, y0), e1 = shadow_margin(o1, y1), e2 = shadow_margin(o2, y2);
+    const float l0 = fminf(o0, y0) - e0, l1 = fminf(o1, y1) - e1, l2 = fminf(o2, y2) - e2;
+    const float h0 = fmaxf(o0, y0) + e0, h1 = fmaxf(o1, y1) + e1, h2 = fmaxf(o2, y2) + e2;
+    const float4* s_box = bt.boxes();
+    return bt.any(l0, l1, l2, h0, h1, h2, [&](int b) {
+        const float4 bmin = s_box[2 * b], bmax = s_box[2 * b + 1];
+        if (bmin.x > h0 || bmax.x < l0 || bmin.y > h1 || bmax.y < l1 || bmin.z > h2 || bmax.z < l2) return false;
+        return slabs_cross(bmin, bmax, i0, i1, i2, q0, q1, q2);
+    });
+}
+}  // namespace
+
 struct ShadeOut {
     float est[3];
     float reward;
@@ -142,27 +185,15 @@ __device__ __forceinline__ ShadeOut shade(const LightRec& L, float x0, float x1,
                 i2 = fdiv(1.0f, seg_dir(fsub(y2, o2)));
     const float q0 = -fmul(o0, i0), q1 = -fmul(o1, i1), q2 = -fmul(o2, i2);
     // Conservative prefilter: a box can only block the segment if it meets the
-    // segment's bounding box widened by del; del exceeds the rounding error of
-    // the slab planes below (a few ulps of |o| + |y|), so no box the exact
+    // segment's bounding box widened by shadow_margin, so no box the exact
     // slab test would report is skipped and the decision is unchanged.
-    const float e0 = 1e-5f * (1.0f + fabsf(o0) + fabsf(y0));
-    const float e1 = 1e-5f * (1.0f + fabsf(o1) + fabsf(y1));
-    const float e2 = 1e-5f * (1.0f + fabsf(o2) + fabsf(y2));
+    const float e0 = shadow_margin(o0, y0), e1 = shadow_margin(o1, y1), e2 = shadow_margin(o2, y2);
     const float4* s_box = bt.boxes();
-    const bool occluded = bt.any(fminf(o0, y0) - e0, fminf(o1, y1) - e1, fminf(o2, y2) - e2, fmaxf(o0, y0) + e0,
-                                 fmaxf(o1, y1) + e1, fmaxf(o2, y2) + e2, [&](int b) {
-        const float4 bmin = s_box[2 * b], bmax = s_box[2 * b + 1];
-        const float ta0 = __fmaf_rn(bmin.x, i0, q0), tb0 = __fmaf_rn(bmax.x, i0, q0);
-        const float ta1 = __fmaf_rn(bmin.y, i1, q1), tb1 = __fmaf_rn(bmax.y, i1, q1);
-        const float ta2 = __fmaf_rn(bmin.z, i2, q2), tb2 = __fmaf_rn(bmax.z, i2, q2);
-        float tn = fmaxf(0.0f, fminf(ta0, tb0));
-        float tf = fminf(kShadowTmax, fmaxf(ta0, tb0));
-        tn = fmaxf(tn, fminf(ta1, tb1));
-        tf = fminf(tf, fmaxf(ta1, tb1));
-        tn = fmaxf(tn, fminf(ta2, tb2));
-        tf = fminf(tf, fmaxf(ta2, tb2));
-        return tn < tf;
-    });
+    auto blocks = [&](int b) { return slabs_cross(s_box[2 * b], s_box[2 * b + 1], i0, i1, i2, q0, q1, q2); };
+    const bool occluded =
+        bt.swapped() ? spanned_box_blocks(bt, o0, o1, o2, y0, y1, y2)
+                     : bt.any(fminf(o0, y0) - e0, fminf(o1, y1) - e1, fminf(o2, y2) - e2, fmaxf(o0, y0) + e0,
+                              fmaxf(o1, y1) + e1, fmaxf(o2, y2) + e2, blocks);
     ShadeOut o;
     const float wx = y0 - x0, wy = y1 - x1, wz = y2 - x2;
     const float d2 = wx * wx + wy * wy + wz * wz;

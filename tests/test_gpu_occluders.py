@@ -1,5 +1,6 @@
 """Occluder sets that the ordinary ones leave out: batches of items
-with different box counts, boxes met at the same distance (marked gpu)."""
+with different box counts, boxes met at the same distance, boxes
+given with minimum and maximum exchanged (marked gpu)."""
 import dataclasses
 
 import numpy as np
@@ -7,7 +8,7 @@ import pytest
 
 from paper_1911_10217_gb300 import scenes
 
-from .gpu_common import params_for
+from .gpu_common import device_scene, params_for
 from .test_gpu_batched import _build
 from .test_gpu_boxes import random_boxes
 from .test_gpu_descent import env as _descent_env  # noqa: F401
@@ -100,3 +101,74 @@ def test_bounce_on_two_boxes_at_the_same_distance(env):
             axes.append(int(np.argmax(np.abs(want[1][:, p]))))
         assert axes == [1, 0]  # the two are at the same distance indeed
     assert tried >= 2
+
+
+def swapped(boxes, seed):
+    """Every other box with minimum and maximum exchanged along some axes."""
+    rng = np.random.default_rng(seed)
+    out = boxes.copy()
+    for b in range(0, len(out), 2):
+        for k in range(3):
+            if rng.uniform() < 0.5:
+                out[b, k], out[b, 3 + k] = boxes[b, 3 + k], boxes[b, k]
+    return out
+
+
+@pytest.mark.parametrize("n", [1, 64, 300])
+def test_bounce_on_boxes_the_other_way_round(env, n):
+    """The slab test takes a box with minimum and maximum exchanged like any other."""
+    O, rll, ctx, torch, dev = env["O"], env["rll"], env["ctx"], env["torch"], env["dev"]
+    boxes = swapped(random_boxes(n), n)
+    rng = np.random.default_rng(4)
+    P = 4001
+    pos = rng.uniform(0.0, 1.0, (3, P)).astype(np.float32)
+    nrm = rng.normal(size=(3, P))
+    nrm = (nrm / np.linalg.norm(nrm, axis=0)).astype(np.float32)
+    want = O.bounce_vertices(pos, nrm, boxes, scenes.ROOM, 9, 2, 50.0)
+    t = lambda a: torch.from_numpy(np.ascontiguousarray(a)).to(dev)  # noqa: E731
+    out = [torch.empty(3, P, device=dev), torch.empty(3, P, device=dev), torch.empty(P, device=dev)]
+    rll.bounce_vertices(ctx, t(pos), t(nrm), t(boxes), scenes.ROOM, 9, 2, 50.0, *out)
+    for got, w in zip(out, want):
+        assert np.array_equal(got.cpu().numpy(), np.asarray(w, np.float32))
+
+
+@pytest.mark.parametrize("axis", [0, 1, 2])
+def test_shadow_of_a_box_the_other_way_round(env, axis):
+    """To the shadow test a box with minimum and maximum exchanged along an axis counts where the segment
+    spans all of it: one from far beyond the room to far before it never does."""
+    rll, ctx, torch, dev = env["rll"], env["ctx"], env["torch"], env["dev"]
+    s = scenes.small_frame_scene()
+    d = device_scene(s, dev)
+    tree = rll.Tree(ctx, d["tri"], d["em"])
+    one = np.array([[.45, .45, .45, .55, .55, .55]], np.float32)  # the bins are cut over this one
+    far = np.array([[-10, -10, -10, 10, 10, 10]], np.float32)
+    far[0, [axis, 3 + axis]] = 10, -10
+    images = []
+    for boxes in (one, np.concatenate([one, far])):
+        b = torch.from_numpy(boxes).to(dev)
+        grid = rll.Grid(ctx, tree, params_for(rll, s))
+        rgb, power = torch.empty(3, s.n_points, device=dev), torch.empty(3, s.n_points, device=dev)
+        rll.sample_and_shade(ctx, grid, tree, d["pos"], d["nrm"], d["alb"], b, 5, 0, 1, rgb)
+        rll.sample_power(ctx, tree, d["pos"], d["nrm"], d["alb"], b, 5, 0, 1, power)
+        images.append((rgb.cpu().numpy(), power.cpu().numpy()))
+    for a, b in zip(*images):
+        assert np.count_nonzero(a) > 100 and np.array_equal(a, b)
+
+
+def test_shadow_of_a_spanned_box(env):
+    """A thin wall given the other way round blocks the segments that cross all of it, like the wall
+    itself; only segments that end inside it (a thousandth of the room) may differ."""
+    rll, ctx, torch, dev = env["rll"], env["ctx"], env["torch"], env["dev"]
+    s = scenes.small_frame_scene()
+    d = device_scene(s, dev)
+    tree = rll.Tree(ctx, d["tri"], d["em"])
+    wall = np.array([[.4995, -1, -1, .5005, 2, 2]], np.float32)
+    images = []
+    for boxes in (wall[:0], wall, wall[:, [3, 1, 2, 0, 4, 5]]):
+        b = torch.from_numpy(np.ascontiguousarray(boxes)).to(dev)
+        rgb = torch.empty(3, s.n_points, device=dev)
+        rll.sample_power(ctx, tree, d["pos"], d["nrm"], d["alb"], b, 5, 0, 1, rgb)
+        images.append(rgb.cpu().numpy())
+    blocked = np.any(images[0] != images[1], axis=0)
+    assert np.mean(blocked) > 0.2
+    assert np.mean(np.all(images[1] == images[2], axis=0)) > 0.99
