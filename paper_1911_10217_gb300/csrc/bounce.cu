@@ -2,8 +2,8 @@
 // ingredient: the cells of a path vertex are sized from its ray footprint,
 // derived from the vertex's area pdf).
 //
-// One thread per shading point x (unit normal n), occluder boxes and their
-// table (box_bins.cuh) staged in shared memory once per block:
+// One thread per shading point x (unit normal n), occluder boxes, and of many
+// their table (box_bins.cuh), staged in shared memory once per block:
 //   a uniform point (a, b) of the unit disk by rejection from the point's
 //   Philox stream (counter (point, frame, draw / 4, 1); pair k = draws 2k,
 //   2k + 1 as 2u - 1; first k < 16 inside the disk, else the centre);
@@ -33,12 +33,18 @@ constexpr int kBounceTries = 16;
 constexpr float kBounceOffset = 1e-4f;
 constexpr float kBounceTmin = 1e-6f;
 constexpr float kPiF = 3.14159265358979323846f;
+// Up to so many boxes are tested in turn, without a table, by a block per 256 points: 1080p bounces
+// take 40 us and 3.5 us a box so, and with the table 103 at one box and 98 to 115 at 16 to 24 boxes
+// (random small ones, large ones, a room's walls), 125 to 138 at 64. In launches of at most a block an
+// SM the table's build counts for more: 64x64 points and 32 boxes 10.9 us without it, 12 to 13 with.
+constexpr int kFewBoxes = 20, kFewBoxesSmall = 32;
 
 __device__ __forceinline__ float fdivr(float a, float b) { return __fdiv_rn(a, b); }
 
-// As many blocks as fit the device, striding over the points: each builds the box table for itself, so
-// that bounces share no table with calls on other streams (path vertices at 720p 415 us a pass with
-// one table a launch and a block per 256 points, 418 so).
+// Many boxes: as many blocks as fit the device, striding over the points; each builds the box table
+// for itself, so that bounces share no table with calls on other streams (path vertices at 720p 415 us
+// a pass with one table a launch and a block per 256 points, 418 so). FEW: see kFewBoxes.
+template <bool FEW>
 __global__ void __launch_bounds__(kBounceThreads)
 k_bounce(const float* __restrict__ pos, const float* __restrict__ nrm, int64_t np, const float* __restrict__ boxes,
          int n_boxes, float r0, float r1, float r2, float r3, float r4, float r5, uint2 key, uint32_t frame,
@@ -46,7 +52,16 @@ k_bounce(const float* __restrict__ pos, const float* __restrict__ nrm, int64_t n
 {
     pdl_begin();
     extern __shared__ float4 s_boxes[];
-    const BoxTable bt = stage_box_table<true>(s_boxes, nullptr, n_boxes, boxes);
+    BoxTable bt{};
+    if constexpr (FEW) {
+        for (int b = threadIdx.x; b < n_boxes; b += blockDim.x) {
+            const float* v = boxes + 6 * b;
+            s_boxes[2 * b] = make_float4(v[0], v[1], v[2], 0.0f);
+            s_boxes[2 * b + 1] = make_float4(v[3], v[4], v[5], 0.0f);
+        }
+    } else {
+        bt = stage_box_table<true>(s_boxes, nullptr, n_boxes, boxes);
+    }
     __syncthreads();
     for (int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; p < np; p += (int64_t)gridDim.x * blockDim.x) {
         const float x[3] = {pos[p], pos[np + p], pos[2 * np + p]};
@@ -98,9 +113,9 @@ k_bounce(const float* __restrict__ pos, const float* __restrict__ nrm, int64_t n
                 axis = k;
             }
         }
-        // The nearest box face in front of it, in up to four segments of the ray, the first an eighth of
-        // the boxes' extent long, each other twice the one before and the last the rest: most rays end in
-        // the first two, near which few boxes are (path vertices at 720p: 465 us a pass with the whole ray
+        // The nearest box face in front of it, of many boxes in up to four segments of the ray, the first
+        // an eighth of the boxes' extent long, each other twice the one before and the last the rest: most
+        // rays end in the first two, near which few boxes are (path vertices at 720p: 465 us a pass with the whole ray
         // at once, now 414). A box whose face is met in a segment meets the segment's
         // bounding box; widened by a margin above the rounding errors of the slab planes and of the
         // segment's ends (a few ulps of the coordinates), it keeps every box that counts. Of boxes met at
@@ -108,7 +123,7 @@ k_bounce(const float* __restrict__ pos, const float* __restrict__ nrm, int64_t n
         // an early segment and is met beyond it shortens the next ones, but is met again in the last,
         // in its turn (its distance is raised by an ulp until then; told apart by their indices at every
         // test instead, or left to the last segment altogether, 1080p bounces took 130 us, now 125).
-        const float4* s_box = bt.boxes();
+        const float4* s_box = FEW ? s_boxes : bt.boxes();
         const float t_wall = t_best;
         auto face = [&](int i) {
             const float4 lo4 = s_box[2 * i], hi4 = s_box[2 * i + 1];
@@ -136,8 +151,10 @@ k_bounce(const float* __restrict__ pos, const float* __restrict__ nrm, int64_t n
             }
             return false;
         };
+        if constexpr (FEW)
+            for (int i = 0; i < n_boxes; ++i) face(i);
         float near = 0.0f, step = 0.125f * bt.extent();
-        for (int seg = 0;; ++seg) {
+        for (int seg = 0; !FEW; ++seg) {
             const bool rest = seg == 3 || !(step > 0.0f) || !(near + step < t_best);
             const float far = rest ? t_best : near + step;
             float lo[3], hi[3];
@@ -192,10 +209,14 @@ extern "C" int rll_bounce_vertices(rll_ctx* ctx, const float* pos, const float* 
         return fail(ctx, RLL_E_INVALID, "NULL point or output array");
     if (n_points == 0) return RLL_OK;
     DeviceGuard g(ctx->device);
-    const size_t smem = n_boxes ? box_table_bytes(n_boxes) : 0;
-    const unsigned blocks = resident_blocks(ctx, k_bounce, n_points, kBounceThreads, smem);
+    const int64_t point_blocks = (n_points + kBounceThreads - 1) / kBounceThreads;
+    const bool few = n_boxes <= (point_blocks <= device_sm_count(ctx->device) ? kFewBoxesSmall : kFewBoxes);
+    const size_t smem = few ? 32 * (size_t)n_boxes : box_table_bytes(n_boxes);
+    auto* kernel = few ? k_bounce<true> : k_bounce<false>;
+    const unsigned blocks = few ? (unsigned)point_blocks
+                                : resident_blocks(ctx, kernel, n_points, kBounceThreads, smem);
     return check_cuda(ctx,
-                      launch_pdl(k_bounce, dim3(blocks), dim3(kBounceThreads), smem, ctx->stream, pos, nrm, n_points,
+                      launch_pdl(kernel, dim3(blocks), dim3(kBounceThreads), smem, ctx->stream, pos, nrm, n_points,
                                  boxes, (int)n_boxes, room[0], room[1], room[2], room[3], room[4], room[5],
                                  make_uint2((uint32_t)seed, (uint32_t)(seed >> 32)), frame, paths_per_tile, out_pos,
                                  out_nrm, out_footprint),

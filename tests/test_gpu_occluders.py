@@ -71,7 +71,7 @@ def test_bounce_on_two_boxes_at_the_same_distance(env):
     f = np.float32
     x, n, seed, frame, P = [0.51, 0.05, 0.5], [0.0, 1.0, 0.0], 9, 2, 4000
     pos, nrm = (np.repeat(np.array(v, f)[:, None], P, 1) for v in (x, n))
-    corners = np.array([[0, 0, 0, .01, .01, .01], [.99, .99, .99, 1, 1, 1]], f)
+    corners = np.tile(np.array([[0, 0, 0, .01, .01, .01], [.99, .99, .99, 1, 1, 1]], f), (20, 1))  # many boxes
     t = lambda a: torch.from_numpy(np.ascontiguousarray(a)).to(dev)  # noqa: E731
     tried = 0
     for p in range(P):
@@ -172,3 +172,22 @@ def test_shadow_of_a_spanned_box(env):
     blocked = np.any(images[0] != images[1], axis=0)
     assert np.mean(blocked) > 0.2
     assert np.mean(np.all(images[1] == images[2], axis=0)) > 0.99
+
+
+@pytest.mark.parametrize("points,n", [(300, 0), (300, 20), (300, 21), (300, 32), (300, 33), (45000, 0), (45000, 1),
+                                      (45000, 20), (45000, 21)])
+def test_bounce_over_few_boxes(env, points, n):
+    """Up to 20 boxes, or 32 in launches of at most a block an SM (38 912 points), are tested in turn;
+    more over the table."""
+    O, rll, ctx, torch, dev = env["O"], env["rll"], env["ctx"], env["torch"], env["dev"]
+    boxes = random_boxes(max(n, 1))[:n]
+    rng = np.random.default_rng(n)
+    pos = rng.uniform(-0.1, 1.1, (3, points)).astype(np.float32)
+    nrm = rng.normal(size=(3, points))
+    nrm = (nrm / np.linalg.norm(nrm, axis=0)).astype(np.float32)
+    want = O.bounce_vertices(pos, nrm, boxes, scenes.ROOM, 9, 2, 50.0)
+    t = lambda a: torch.from_numpy(np.ascontiguousarray(a)).to(dev)  # noqa: E731
+    out = [torch.empty(3, points, device=dev), torch.empty(3, points, device=dev), torch.empty(points, device=dev)]
+    rll.bounce_vertices(ctx, t(pos), t(nrm), t(boxes), scenes.ROOM, 9, 2, 50.0, *out)
+    for got, w in zip(out, want):
+        assert np.array_equal(got.cpu().numpy(), np.asarray(w, np.float32))
