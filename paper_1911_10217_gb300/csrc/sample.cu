@@ -40,7 +40,7 @@ __global__ void __launch_bounds__(THREADS, MINB) k_sample(SampleArgs a)
 {
     pdl_begin();
     extern __shared__ float4 s_boxes[];
-    const BoxTable bt = stage_box_table<SPLIT != LOOP>(s_boxes, a.box_table, a.n_boxes, a.boxes);
+    const BoxTable bt = stage_box_table<SPLIT != LOOP, true>(s_boxes, a.box_table, a.n_boxes, a.boxes);
     if constexpr (SPLIT == LANES) {
         __shared__ float s_est[THREADS / 32][kWarpEst];
         __syncthreads();
@@ -71,7 +71,7 @@ __global__ void __launch_bounds__(THREADS, MINB) k_sample(SampleArgs a)
 // each builds heap and box table once and the launch needs no table of the context's (311 -> 292 us).
 constexpr int kPowerLevels = 9;  // 2 KB beside the box table of up to 45 KB
 
-__global__ void __launch_bounds__(kThreads) k_sample_power(SampleArgs a, int32_t* light_out)
+__global__ void __launch_bounds__(kThreads, 4) k_sample_power(SampleArgs a, int32_t* light_out)
 {
     pdl_begin();
     extern __shared__ float4 s_boxes[];

@@ -1,6 +1,7 @@
 """Occluder sets that the ordinary ones leave out: batches of items
 with different box counts, boxes met at the same distance, boxes
-given with minimum and maximum exchanged (marked gpu)."""
+given with minimum and maximum exchanged, few boxes, boxes that reach far out
+of the room (marked gpu)."""
 import dataclasses
 
 import numpy as np
@@ -11,7 +12,7 @@ from paper_1911_10217_gb300 import scenes
 from .gpu_common import device_scene, params_for
 from .test_gpu_batched import _build
 from .test_gpu_boxes import random_boxes
-from .test_gpu_descent import env as _descent_env  # noqa: F401
+from .test_gpu_descent import check, env as _descent_env  # noqa: F401
 
 pytestmark = pytest.mark.gpu
 
@@ -188,6 +189,46 @@ def test_bounce_over_few_boxes(env, points, n):
     want = O.bounce_vertices(pos, nrm, boxes, scenes.ROOM, 9, 2, 50.0)
     t = lambda a: torch.from_numpy(np.ascontiguousarray(a)).to(dev)  # noqa: E731
     out = [torch.empty(3, points, device=dev), torch.empty(3, points, device=dev), torch.empty(points, device=dev)]
+    rll.bounce_vertices(ctx, t(pos), t(nrm), t(boxes), scenes.ROOM, 9, 2, 50.0, *out)
+    for got, w in zip(out, want):
+        assert np.array_equal(got.cpu().numpy(), np.asarray(w, np.float32))
+
+
+def stretched_boxes(kind, n):
+    """n boxes of which a few lie or reach far out of the room."""
+    b = random_boxes(n)
+    far = np.float32(3e38 if kind == "huge" else np.inf)
+    if kind == "slab":
+        b[-1] = (-100, -1.1, -100, 100, -1, 100)
+    elif kind == "walls":
+        b[-4:] = [(-9, -9, -9, 9, -8.9, 9), (-9, 8.9, -9, 9, 9, 9), (-9, -9, -9, -8.9, 9, 9), (8.9, -9, -9, 9, 9, 9)]
+    elif kind in ("huge", "endless"):
+        b[-1], b[0] = (-far, .9, -far, far, far, far), (-far, -far, -far, -.2, far, far)
+    elif kind == "steps":  # ever farther
+        for i in range(min(n // 4, 20)):
+            b[i] += np.float32(4.0 ** i)
+    elif kind == "alike":  # ends that no bins tell apart, but for two
+        b[2:] = (.4, .4, .4, .4, .6, .6)
+    return b
+
+
+@pytest.mark.parametrize("n", [64, 300])
+@pytest.mark.parametrize("kind", ["slab", "walls", "huge", "endless", "steps", "alike"])
+def test_bins_that_few_boxes_would_stretch(env, kind, n):
+    """The bins are cut over the range of most boxes: samples and vertices against the oracle, which
+    tests every box."""
+    O, rll, ctx, torch, dev = env["O"], env["rll"], env["ctx"], env["torch"], env["dev"]
+    boxes = stretched_boxes(kind, n)
+    check(env, dataclasses.replace(scenes.tiny_scene(), boxes=boxes), frames=1, spp=2)
+    rng = np.random.default_rng(7)
+    P = 3001
+    pos = rng.uniform(-0.3, 1.3, (3, P)).astype(np.float32)
+    nrm = rng.normal(size=(3, P))
+    nrm[:, :64] = np.eye(3)[:, rng.integers(0, 3, 64)]
+    nrm = (nrm / np.linalg.norm(nrm, axis=0)).astype(np.float32)
+    want = O.bounce_vertices(pos, nrm, boxes, scenes.ROOM, 9, 2, 50.0)
+    t = lambda a: torch.from_numpy(np.ascontiguousarray(a)).to(dev)  # noqa: E731
+    out = [torch.empty(3, P, device=dev), torch.empty(3, P, device=dev), torch.empty(P, device=dev)]
     rll.bounce_vertices(ctx, t(pos), t(nrm), t(boxes), scenes.ROOM, 9, 2, 50.0, *out)
     for got, w in zip(out, want):
         assert np.array_equal(got.cpu().numpy(), np.asarray(w, np.float32))
