@@ -116,9 +116,21 @@ struct BoxTable {
         const unsigned long long* e2 = mask + (5 * bins + box_bin_lo(__fmaf_rn(lo2, sc.z, of.z), bins)) * words;
         for (int w = 0; w < words; ++w) {
             unsigned long long m = b0[w] & e0[w] & b1[w] & e1[w] & b2[w] & e2[w];
-            while (m) {
-                if (test(64 * w + __ffsll((long long)m) - 1)) return true;
-                m &= m - 1;
+            // the word's halves in turn: a 64-bit find-first and clear take twice the instructions, which
+            // tells where most boxes are candidates (52 of 64 boxes in one spot of the room, 1080p:
+            // sampling 457 -> 429 us, energy sampler 269 -> 241, bounces 239 -> 218; the walled room 320,
+            // 88 -> 89 and 126 -> 120)
+            uint32_t cur = (uint32_t)m, next = (uint32_t)(m >> 32);
+            int first = 64 * w + 31;
+            while (cur | next) {
+                if (cur == 0u) {
+                    cur = next;
+                    next = 0u;
+                    first += 32;
+                }
+                const uint32_t bit = cur & (0u - cur);
+                if (test(first - __clz((int)bit))) return true;
+                cur ^= bit;
             }
         }
         return false;
