@@ -55,12 +55,9 @@ void free_tree(rll_tree* t)
 {
     if (!t) return;
     cudaFree(t->nodes);
-    cudaFree(t->pairs);
     if (t->tail_tex) cudaDestroyTextureObject(t->tail_tex);
-    cudaFree(t->tails);
-    cudaFree(t->quads);
     if (t->quad_tex) cudaDestroyTextureObject(t->quad_tex);
-    cudaFree(t->quad_tails);
+    cudaFree(t->records);
     cudaFree(t->lights);
     cudaFree(t->perm);
     cudaFree(t->left);

@@ -53,6 +53,7 @@ struct rll_tree {
     int device = 0;
     int64_t n = 0;
     rll::NodeRec* nodes = nullptr;   // [2n-1] every node
+    void* records = nullptr;         // one allocation: quads, pairs, quad_tails, tails
     rll::PairRec* pairs = nullptr;   // [n-1] geometry of both children of internal i, interleaved
     rll::PairTail* tails = nullptr;  // [n-1] their powers and ids
     cudaTextureObject_t tail_tex = 0; // tails as float4 texels (n > 1)

@@ -630,10 +630,19 @@ int build_tree(rll_ctx* ctx, const float* tri, const float* emission, int64_t n,
     e = cudaMalloc((void**)&(ptr), (bytes) > 0 ? (bytes) : 64);               \
     if (e != cudaSuccess) return check_cuda(ctx, e, "cudaMalloc(tree)");
     RLL_ALLOC(t->nodes, sizeof(NodeRec) * nn);
-    RLL_ALLOC(t->pairs, sizeof(PairRec) * (n - 1));
-    RLL_ALLOC(t->tails, sizeof(PairTail) * (n - 1));
-    RLL_ALLOC(t->quads, sizeof(QuadRec) * (n - 1));
-    RLL_ALLOC(t->quad_tails, sizeof(QuadTail) * (n - 1));
+    {  // the descent records in one allocation: of a megabyte and more, each one takes as long as several of
+       // the kernels here (a tree of 64K lights 609 us and 264 to free it with four, now 494 and 178)
+        const int64_t bytes[4] = {(int64_t)sizeof(QuadRec) * (n - 1), (int64_t)sizeof(PairRec) * (n - 1),
+                                  (int64_t)sizeof(QuadTail) * (n - 1), (int64_t)sizeof(PairTail) * (n - 1)};
+        int64_t at[5] = {0};
+        for (int k = 0; k < 4; ++k) at[k + 1] = (at[k] + bytes[k] + 511) & ~(int64_t)511;  // texture alignment
+        RLL_ALLOC(t->records, at[4]);
+        char* base = static_cast<char*>(t->records);
+        t->quads = reinterpret_cast<QuadRec*>(base);
+        t->pairs = reinterpret_cast<PairRec*>(base + at[1]);
+        t->quad_tails = reinterpret_cast<QuadTail*>(base + at[2]);
+        t->tails = reinterpret_cast<PairTail*>(base + at[3]);
+    }
     RLL_ALLOC(t->lights, sizeof(LightRec) * n);
     RLL_ALLOC(t->perm, sizeof(uint32_t) * n);
     RLL_ALLOC(t->left, sizeof(int32_t) * (n - 1));
