@@ -151,7 +151,8 @@ template <int P, int MODE>
 cudaError_t launch_m(const SampleArgs& a, bool dbg, int minb, cudaStream_t s)
 {
     if (dbg) return launch<P, MODE, true, LOOP, 256, 3>(a, s);
-    if (a.warp_points) return launch<P, MODE, false, LANES, 128, 8>(a, s);
+    if (a.warp_points)
+        return minb == 4 ? launch<P, MODE, false, LANES, 128, 8>(a, s) : launch<P, MODE, false, LANES, 128, 6>(a, s);
     if (a.spp == 1)
         return minb == 4 ? launch<P, MODE, false, ONE, 128, 8>(a, s) : launch<P, MODE, false, ONE, 128, 6>(a, s);
     return minb == 4 ? launch<P, MODE, false, LOOP, 128, 8>(a, s) : launch<P, MODE, false, LOOP, 128, 6>(a, s);

@@ -70,3 +70,10 @@ def test_a_lane_a_sample(env, points, spp):  # noqa: F811
 def test_one_sample_a_point_and_box_tables(env, points, spp, boxes, mode):  # noqa: F811
     """At most 64 boxes and one wave of blocks (155 648 points): each block builds the boxes' table."""
     check_plain(env, scene_of(points, spp, boxes), mode=mode)
+
+
+@pytest.mark.parametrize("points,spp,mode", [(5000, 9, "descent"), (700, 40, "descent2"), (5000, 1, "descent"),
+                                             (90000, 4, "uniform")])
+def test_forms_of_the_larger_register_budget(env, points, spp, mode):  # noqa: F811
+    """sample_min_blocks = 3 holds for every split of the samples."""
+    check_plain(env, scene_of(points, spp), option=("sample_min_blocks", 3), mode=mode)
