@@ -37,9 +37,9 @@ UNIT = "light samples/s"
 PEAKS_FALLBACK = {"hbm_gbs": 6800.0, "bf16_tflops": 1900.0}
 SM_COUNT = 152
 # DRAM bytes (read + write) of one k_sample launch on this workload, from one ncu capture of it
-# (76.23 MB read + 15.93 MB written; kernel as of commit c41eaaf); None whenever the sampling
+# (76.29 MB read + 15.69 MB written; kernel as of commit 728d662); None whenever the sampling
 # kernel has changed since that capture
-K_SAMPLE_DRAM_BYTES = 92.16e6
+K_SAMPLE_DRAM_BYTES = 91.98e6
 FP32_LANES_PER_SM = 128
 
 
@@ -1053,7 +1053,7 @@ def main():
         hbm_ach = bytes_per_sample() * n_sample / t_s / 1e9
         learn_bytes = learn_step_bytes(n_sample, n_touched, grid.M)
         t_l = statistics.mean(t_learn) * 1e-3
-        # our kernels per step: the box sort and sampling = 2; learning: count, claim, scatter, the warp,
+        # our kernels per step: the box table and sampling = 2; learning: count, claim, scatter, the warp,
         # two-warp and block paths (one launch), the sorting block path = 5; split-collapse 1 unless
         # fused into learning (an ncu launch list of the pass shows them)
         launches_per_step = 2 + 5 + (1 if args.separate_split else 0)

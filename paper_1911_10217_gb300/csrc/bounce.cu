@@ -34,9 +34,10 @@ constexpr float kBounceOffset = 1e-4f;
 constexpr float kBounceTmin = 1e-6f;
 constexpr float kPiF = 3.14159265358979323846f;
 // Up to so many boxes are tested in turn, without a table, by a block per 256 points: 1080p bounces
-// take 40 us and 3.5 us a box so, and with the table 103 at one box and 98 to 115 at 16 to 24 boxes
-// (random small ones, large ones, a room's walls), 125 to 138 at 64. In launches of at most a block an
-// SM the table's build counts for more: 64x64 points and 32 boxes 10.9 us without it, 12 to 13 with.
+// take 40 us and 3.5 us a box so, and with the table 101 at one box, 97 to 107 at 16, 99 to 117 at 20
+// and 103 to 124 at 24 boxes (random small ones, large ones, a room's walls), 122 to 129 at 64. In
+// launches of at most a block an SM the table's build counts for more: 64x64 points and 24 boxes 10.9
+// us without it, 10.9 to 15 with; 32 boxes 10.9, and 10.9 to 13.
 constexpr int kFewBoxes = 20, kFewBoxesSmall = 32;
 
 __device__ __forceinline__ float fdivr(float a, float b) { return __fdiv_rn(a, b); }
