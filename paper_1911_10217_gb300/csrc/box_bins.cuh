@@ -152,8 +152,7 @@ __device__ __forceinline__ float box_upper(const float* v, int k) { return v[3 +
 // had lost the table's gain and more: 1080p, 64 boxes and that slab, by the loops that the table
 // replaced / by bins over the whole extent / so: sampling 439 / 431 / 331 us, energy sampler 177 / 238 /
 // 95, bounces 269 / 376 / 139; 1 024 boxes and the slab 2 500 / 3 643 / 2 006, 2 016 / 3 410 / 1 667 and
-// 3 665 / 5 300 / 1 236. Boxes without such a one take one step, which finds nothing: 64x64 points
-// 33.5 -> 34.1 us a pass, 1080p passes equal.
+// 3 665 / 5 300 / 1 236. Boxes without such a one take one step, which finds nothing (1080p passes equal).
 __device__ __forceinline__ bool narrow_bins(const uint32_t* begins, const uint32_t* ends, int bins, int words, int n,
                                             int most, float* scale, float* off)
 {
@@ -190,6 +189,11 @@ __device__ __forceinline__ bool narrow_bins(const uint32_t* begins, const uint32
     return false;
 }
 constexpr int kMaxNarrow = 12;  // steps, of 2 to 32 times each
+// Up to so many boxes keep the whole extent: testing all of them costs less than the look at the bins
+// in a small launch (64x64 points, 8 boxes: 33.6 us a pass with it, 32.9 without; 1080p, 14 boxes and the
+// slab: sampling 320 and 330 us, energy sampler 95 and 106, by loops over all boxes 400 and 146; 16 boxes
+// and 6 distant walls are narrowed: 321 and 95, not narrowed 345 and 122).
+constexpr int kFewToNarrow = 16;
 
 // Builds the table of n (1 .. kMaxBoxes) boxes [n][6] into out, by a whole block of 96 to 256
 // threads; s_mask: its masks in shared memory, or a scratch copy of them there (box_mask_bytes).
@@ -252,6 +256,7 @@ __device__ __forceinline__ void build_box_table(const float* __restrict__ boxes,
             atomicOr(&s_mask[((2 * k + 1) * bins + j1) * words + (b >> 5)], 1u << (b & 31));
         }
         __syncthreads();
+        if (n <= kFewToNarrow) break;
         bool again = false;
         if (!wide) {
             const uint32_t* begins = s_mask + 2 * warp * bins * words;

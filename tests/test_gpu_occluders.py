@@ -212,7 +212,7 @@ def stretched_boxes(kind, n):
     return b
 
 
-@pytest.mark.parametrize("n", [64, 300])
+@pytest.mark.parametrize("n", [16, 17, 64, 300])
 @pytest.mark.parametrize("kind", ["slab", "walls", "huge", "endless", "steps", "alike"])
 def test_bins_that_few_boxes_would_stretch(env, kind, n):
     """The bins are cut over the range of most boxes: samples and vertices against the oracle, which
